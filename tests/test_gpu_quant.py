@@ -365,3 +365,20 @@ def test_prepare_weight(N, K, g, rotate):
     check_scales(scale.cpu().numpy(), ref["scale"], w.astype(np.float64), g, rotate, what="weight scale")
     # Row sums are exact integers of the GPU's own codes.
     np.testing.assert_array_equal(rowsum.cpu().numpy(), qg.reshape(N, K // g, g).sum(axis=2).T)
+
+
+@pytest.mark.parametrize("N,K,g", [(1, 32, 32), (33, 96, 32), (65, 192, 64), (31, 384, 128), (32, 8192, 8192),
+                                   (70, 5120, 512)])
+def test_prepare_weight_block_widths(N, K, g):
+    """The repacking warps' shares: one 16-byte chunk per offset block (g = 32) up to 256 (g = 8192), units that do
+    not fill the last CTA, and ragged rows. Codes, sums and zeroed padding are exact on grid-valued weights."""
+    rng = np.random.default_rng(N + K + g)
+    q = rng.integers(-7, 8, size=(N, K))
+    q[:, 0] = 7
+    w = (q * 2.0 ** -6).astype(np.float32)
+    codes, scale, rowsum = Q.prepare_weight(torch.from_numpy(w).cuda(), g, rotate=False)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(weight_q(codes, N, K), q)
+    np.testing.assert_array_equal(rowsum.cpu().numpy(), q.reshape(N, K // g, g).sum(axis=2).T)
+    full = codes.cpu().numpy()
+    assert not O.untile_codes(full, full.shape[0], K)[N:].any()
