@@ -126,11 +126,8 @@ def test_oracle_codes_through_gemm():
     # accumulator; and a K that is not a multiple of the 4-k-tile bulk copies.
     (9, 1024, 28672, 1024, "bf16", None),
     (17, 1920, 640, 128, "f16", None),
-    # Few-token form (T <= 4, dp4a on the CUDA cores): every token count class (1, 2, 4 with
-    # 3 padded), K = 1056 (33 chunks: the eighths of K are uneven and the last warp has none),
-    # K = 11008 at 4 tokens (43 KB of unpacked activations, 43 offset blocks), and a K whose
-    # unpacked activations exceed its budget (4 x 32768 bytes: the tensor-core form). Then the
-    # decode kernel at its smallest token counts (5 to 8: 11 to 14 padded MMA columns).
+    # Few-token form: one to eight tokens, K = 1056 (33 chunks: the eighths of K are uneven and
+    # the last warps have none), 43 offset blocks, and a long K.
     (1, 1024, 300, 256, "f32", None),
     (2, 4096, 1000, 4096, "f16", 1000),
     (3, 1056, 520, 32, "bf16", None),
@@ -143,6 +140,22 @@ def test_oracle_codes_through_gemm():
 ])
 def test_layers(T, K, N, g, out_dt, ldo):
     _check_layer(T, K, N, g, out_dt, ldo=ldo, seed=T + K)
+
+
+@pytest.mark.parametrize("T,K,N,g,out_dt", [
+    (1, 32, 40, 32, "f32"),          # one chunk: a single warp has a k-step, of one chunk
+    (8, 160, 33, 32, "bf16"),        # five chunks: a step with one chunk; one channel past a row block
+    (9, 1056, 64, 32, "f16"),        # 9 to 16 tokens; 33 offset blocks in shared memory
+    (16, 4096, 31, 32, "f32"),       # 128 offset blocks: read from global memory
+    (17, 2048, 96, 32, "f32"),       # 17 to 32 tokens, 64 offset blocks: the staging limit
+    (32, 2080, 100, 32, "bf16"),     # 65 offset blocks: past it
+    (5, 512, 9856, 512, "bf16"),     # more than two weight blocks per SM: the three-CTA instantiation
+    (31, 4096, 256, 1024, "f16"),
+])
+def test_few_token_form(T, K, N, g, out_dt):
+    """The few-token kernel at the edges of its k-steps, token tiles, offset staging and CTA budgets."""
+    ldo = (N + 7) // 8 * 8
+    _check_layer(T, K, N, g, out_dt, ldo=ldo, seed=T * 7 + K)
 
 
 def test_no_rotation_site():
@@ -188,7 +201,7 @@ def test_accumulator_exact_at_largest_k():
 @pytest.mark.parametrize("T", [1, 8, 96])
 def test_accumulator_exact_at_maximum_k(T):
     """K = 65536, the largest the ABI takes, with every code at +-7, through each form of the
-    linear (CUDA-core at 1 token, the decode kernel at 8, the pair kernel at 96): the largest
+    linear (the few-token form at 1 and 8 tokens, the pair kernel at 96): the largest
     sum, 15 * 7 * 65536 < 2^24, stays exact."""
     N, K, g = 256, 65536, 8192
     qa = np.full((T, K), 7, dtype=np.int64)
