@@ -31,7 +31,7 @@
 // reads and 16 KB of B stores, against 512 cycles of MMA work.
 //
 // Warp roles per CTA (21 warps):
-//   warp 0       TMEM allocation; in the leader CTA, lane 0 issues the MMAs
+//   warp 0       TMEM allocation; in the leader CTA, an elected lane issues the MMAs
 //   warps 1-8    A converters: two per 32-lane quarter of TMEM, alternating k-tiles
 //   warps 9-16   B converters: two per 32-row group, alternating k-tiles
 //   warps 17-20  epilogue (one per TMEM quarter, all 256 columns)
@@ -271,31 +271,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
 
   if (warp == 0) {
     // ---------------- MMA issuer (leader CTA) ----------------
-    if (rank == 0 && lane == 0) {
+    // The whole warp runs the loop; an elected lane issues (elect_one).
+    if (rank == 0) {
+      const uint64_t desc0 = smem_desc_sw128(base + kOffB);
       int s = 0, phase = 0, lt = 0;  // stage and phase parity of the next k-tile
-      for (int tile = cluster; tile < num_tiles && !*abort; tile += clusters, ++lt) {
-        if (!wait_cluster(acc_empty, (lt & 1) ^ 1, abort)) break;
+      for (int tile = cluster; tile < num_tiles; tile += clusters, ++lt) {
+        if (!__all_sync(0xFFFFFFFFu, wait_cluster(acc_empty, (lt & 1) ^ 1, abort))) break;
         tc_fence_after();
         bool ok = true;
         for (int kt = 0; kt < nk; ++kt) {
-          if (!wait_cluster(full(s), phase, abort)) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xFFFFFFFFu, wait_cluster(full(s), phase, abort));
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t b_addr = base + kOffB + s * kBStage;
+          if (elect_one()) {
+            const uint64_t desc = desc0 + static_cast<uint32_t>(s * (kBStage >> 4));
 #pragma unroll
-          for (int kk = 0; kk < BK / 32; ++kk) {
-            mma2_ts(tmem, tmem + kACol0 + s * kAColsPerStage + 8 * kk, smem_desc_sw128(b_addr + 32 * kk), kIdesc,
-                    (kt | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < BK / 32; ++kk)
+              mma2_ts(tmem, tmem + kACol0 + s * kAColsPerStage + 8 * kk, desc + 2 * kk, kIdesc, (kt | kk) != 0 ? 1u : 0u);
+            mma2_commit_both(empty(s));
           }
-          mma2_commit_both(empty(s));
+          __syncwarp();
           if (++s == kStages) {
             s = 0;
             phase ^= 1;
           }
         }
-        mma2_commit_both(acc_full);
+        if (elect_one()) mma2_commit_both(acc_full);
+        __syncwarp();
         mma_tiles = lt + 1;
         if (!ok) break;
       }

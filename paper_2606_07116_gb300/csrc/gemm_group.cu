@@ -30,7 +30,7 @@
 // A stages, and each scaler thread's 64 running sums in its registers.
 //
 // Warp roles per CTA (15 warps, so up to 128 registers per thread):
-//   warp 0       TMEM allocation; in the leader CTA, lane 0 issues the MMAs
+//   warp 0       TMEM allocation; in the leader CTA, an elected lane issues the MMAs
 //   warps 1-4    A converters: one per 32-lane TMEM quarter, every k-tile
 //   warps 5-6    B converters: one per 32-row group (64 rows of B per CTA)
 //   warps 7-14   scalers and epilogue, two per TMEM quarter (64 columns each);
@@ -212,32 +212,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 
   if (warp == 0) {
     // ---------------- MMA issuer (leader CTA) ----------------
-    if (rank == 0 && lane == 0) {
+    // The whole warp runs the loop; an elected lane issues (elect_one).
+    if (rank == 0) {
+      const uint64_t desc0 = smem_desc_sw128(base);
       int s = 0, phase = 0;
       uint32_t j = 0;
-      for (int tile = cluster; tile < num_tiles && !*abort; tile += clusters) {
-        bool ok = true;
+      bool ok = true;
+      for (int tile = cluster; tile < num_tiles && ok; tile += clusters) {
         for (int kt = 0; kt < nk; ++kt, ++j) {
           const uint32_t b = j & 1u, use = j >> 1;
-          if (!wait_cluster(pempty(b), (use & 1u) ^ 1u, abort) || !wait_cluster(full(s), phase, abort)) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xFFFFFFFFu, wait_cluster(pempty(b), (use & 1u) ^ 1u, abort) &&
+                                           wait_cluster(full(s), phase, abort));
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t b_addr = base + s * kGBStage;
+          if (elect_one()) {
+            const uint64_t desc = desc0 + static_cast<uint32_t>(s * (kGBStage >> 4));
 #pragma unroll
-          for (int kk = 0; kk < GBK / 32; ++kk)
-            mma2_ts(tmem + kPCol0 + b * GBN, tmem + kGACol0 + s * kGAColsPerStage + 8 * kk,
-                    smem_desc_sw128(b_addr + 32 * kk), kGIdesc, kk != 0 ? 1u : 0u);
-          mma2_commit_both(empty(s));
-          mma2_commit_both(pfull(b));
+            for (int kk = 0; kk < GBK / 32; ++kk)
+              mma2_ts(tmem + kPCol0 + b * GBN, tmem + kGACol0 + s * kGAColsPerStage + 8 * kk, desc + 2 * kk, kGIdesc,
+                      kk != 0 ? 1u : 0u);
+            mma2_commit_both(empty(s));
+            mma2_commit_both(pfull(b));
+          }
+          __syncwarp();
           mma_groups = j + 1;
           if (++s == kGStages) {
             s = 0;
             phase ^= 1;
           }
         }
-        if (!ok) break;
       }
     }
   } else if (warp < kGFirstSc) {

@@ -538,21 +538,25 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      int committed = -1;
-      if (mbar_wait(bar_b, 0, abort)) {
-        for (int i = 0; i < n_local; ++i) {
-          const int s = i % L::kSlots, x = i % kAcc;
-          if (!mbar_wait(full0 + 8 * s, (i / L::kSlots) & 1, abort)) break;
-          if (i >= kAcc && !mbar_wait(tempty0 + 8 * x, ((i / kAcc) - 1) & 1, abort)) break;
-          tc_fence_after();
-          const uint32_t at = ring + s * kOpBytes, acc = tmem + x * L::kAccCols;
+    // The whole warp runs the loop; an elected lane issues (elect_one).
+    const uint64_t b_desc = smem_desc_sw128(b_base), r_desc = smem_desc_sw128(ring);
+    int committed = -1;
+    if (__all_sync(0xFFFFFFFFu, mbar_wait(bar_b, 0, abort))) {
+      for (int i = 0; i < n_local; ++i) {
+        const int s = i % L::kSlots, x = i % kAcc;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8 * s, (i / L::kSlots) & 1, abort) &&
+                                         (i < kAcc || mbar_wait(tempty0 + 8 * x, ((i / kAcc) - 1) & 1, abort))))
+          break;
+        tc_fence_after();
+        const uint32_t acc = tmem + x * L::kAccCols;
+        const uint64_t at = r_desc + static_cast<uint32_t>(s * (kOpBytes >> 4));
+        if (elect_one()) {
           if constexpr (REFLECT) {
 #pragma unroll
             for (int kk = 0; kk < kHd / 16; ++kk) {
               const uint32_t koff = (kk & 3) * 32;
-              mma_bf16(acc, smem_desc_sw128(at + (kk >> 2) * kAtomBytes + koff),
-                       smem_desc_sw128(b_base + (kk >> 2) * kRefAtom + koff), L::kIdesc, kk != 0 ? 1u : 0u);
+              mma_bf16(acc, at + (((kk >> 2) * kAtomBytes + koff) >> 4), b_desc + (((kk >> 2) * kRefAtom + koff) >> 4),
+                       L::kIdesc, kk != 0 ? 1u : 0u);
             }
           } else {
 #pragma unroll
@@ -560,22 +564,22 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
 #pragma unroll
               for (int kk = 0; kk < kHd / 16; ++kk) {
                 const uint32_t koff = (kk >> 2) * kAtomBytes + (kk & 3) * 32;
-                mma_bf16(acc, smem_desc_sw128(at + koff), smem_desc_sw128(b_base + sp * kOpBytes + koff), L::kIdesc,
+                mma_bf16(acc, at + (koff >> 4), b_desc + ((sp * kOpBytes + koff) >> 4), L::kIdesc,
                          (sp | kk) != 0 ? 1u : 0u);
               }
           }
           if constexpr (!kStage) mma_commit(empty0 + 8 * s);  // the tile buffer is free once these MMAs are done
           mma_commit(tfull0 + 8 * x);
-          committed = i;
         }
+        __syncwarp();
+        committed = i;
       }
-      if (*abort && committed >= 0) {
-        // MMAs complete in issue order: wait (bounded) for the last commit
-        // before tensor memory is released.
-        const long long c0 = clock64();
-        while (!mbar_try_wait(tfull0 + 8 * (committed % kAcc), (committed / kAcc) & 1) &&
-               clock64() - c0 < kWaitCycles) {
-        }
+    }
+    if (__any_sync(0xFFFFFFFFu, *abort) && committed >= 0) {
+      // MMAs complete in issue order: wait (bounded) for the last commit
+      // before tensor memory is released.
+      const long long c0 = clock64();
+      while (!mbar_try_wait(tfull0 + 8 * (committed % kAcc), (committed / kAcc) & 1) && clock64() - c0 < kWaitCycles) {
       }
     }
     __syncwarp();

@@ -448,33 +448,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      bool issued = false;
-      for (int n = 0; n < n_local; ++n) {
-        bool ok = true;
-        for (int c = 0; c < 4; ++c) {
-          // Chunk c (slabs 2 c, 2 c + 1) writes column slots 4 c .. 4 c + 3: each
-          // must have been read by the previous tile's second sweep.
-          ok = mbar_wait(full0 + 16 * c, n & 1, abort) && mbar_wait(full0 + 16 * c + 8, n & 1, abort);
-          for (int q = 4 * c; ok && n > 0 && q < 4 * c + 4; ++q) ok = mbar_wait(tempty0 + 8 * q, (n - 1) & 1, abort);
-          if (!ok) break;
-          tc_fence_after();
+    // The whole warp runs the loop; an elected lane issues (elect_one).
+    const uint64_t a_desc = smem_desc_sw128(a_s), b_desc = smem_desc_sw128(b_s);
+    bool issued = false;
+    for (int n = 0; n < n_local; ++n) {
+      bool ok = true;
+      for (int c = 0; c < 4; ++c) {
+        // Chunk c (slabs 2 c, 2 c + 1) writes column slots 4 c .. 4 c + 3: each
+        // must have been read by the previous tile's second sweep.
+        ok = mbar_wait(full0 + 16 * c, n & 1, abort) && mbar_wait(full0 + 16 * c + 8, n & 1, abort);
+        for (int q = 4 * c; ok && n > 0 && q < 4 * c + 4; ++q) ok = mbar_wait(tempty0 + 8 * q, (n - 1) & 1, abort);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            mma_bf16(tmem + 128 * c, smem_desc_sw128(a_s + (2 * c + (kk >> 2)) * kSlabBytes + 32 * (kk & 3)),
-                     smem_desc_sw128(b_s + (kk >> 2) * kBSlab + 32 * (kk & 3)), kIdesc, kk);
-          issued = true;
+            mma_bf16(tmem + 128 * c,
+                     a_desc + static_cast<uint32_t>(((2 * c + (kk >> 2)) * kSlabBytes + 32 * (kk & 3)) >> 4),
+                     b_desc + static_cast<uint32_t>(((kk >> 2) * kBSlab + 32 * (kk & 3)) >> 4), kIdesc, kk);
           mma_commit(empty0 + 16 * c);  // slabs 2 c and 2 c + 1 may take the next tile
           mma_commit(empty0 + 16 * c + 8);
+          if (c == 3) mma_commit(tfull);
         }
-        if (!ok) break;
-        mma_commit(tfull);
+        __syncwarp();
+        issued = true;
       }
-      if (*abort && issued) {
-        // MMAs complete in issue order: one more commit tracks them all.
-        mma_commit(done);
-        mbar_wait_teardown(done, 0);
-      }
+      if (!ok) break;
+    }
+    if (__any_sync(0xFFFFFFFFu, *abort) && issued) {
+      // MMAs complete in issue order: one more commit tracks them all.
+      if (elect_one()) mma_commit(done);
+      __syncwarp();
+      mbar_wait_teardown(done, 0);
     }
     __syncwarp();
   } else {
