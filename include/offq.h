@@ -542,9 +542,9 @@ int offq_prepare_weight_mx(const void* w, int dtype, int64_t N, int64_t K, int32
 /*
  * offq_mx_linear -- the W4A4 linear of MXFP4 operands:
  *   y[t][n] = s_w[n] * ( s_a[t] * sum_k A[t][k] W[n][k] + sum_b o[t][b] R[b][n] ),
- * A = value(e_a) * 2^sh_a and W = value(e_w) * 2^sh_w, each an exact E4M3 value,
- * multiplied on the tensor cores (kind::f8f6f4) with fp32 accumulation,
- * s_a / s_w the row scales. Arguments as offq_w4a4_linear (no acc_debug), plus
+ * A = value(e_a) * 2^sh_a and W = value(e_w) * 2^sh_w, multiplied as block-scaled
+ * FP4 on the tensor cores (kind::mxf4: E2M1 codes, 2^sh as the block's UE8M0
+ * scale; exact products) with fp32 accumulation, s_a / s_w the row scales. Arguments as offq_w4a4_linear (no acc_debug), plus
  * the shift buffers; K a multiple of 128 and of g.
  */
 int offq_mx_linear(const uint8_t* a_codes, const uint8_t* a_shifts, const float* a_scale, const float* a_offset,

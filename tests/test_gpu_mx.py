@@ -179,3 +179,36 @@ def test_mx_gemm_llama2_7b_gate_sampled():
     """The bench's gate projection (2048 x 4096 -> 11008) on sampled rows."""
     rows = np.unique(np.concatenate([W.unit_index_sample(2048, 48, seed=92), [0, 2047]]))
     _check_mx_layer(2048, 4096, 11008, 4096, "bf16", False, seed=93, rows=rows, n_out=4, mult=100.0)
+
+
+@pytest.mark.parametrize("T,K,N,g,out_dt,rotate", [
+    (1, 128, 8, 128, "f32", False),         # one k-tile: half a stage; one row, a few columns
+    (128, 384, 192, 128, "bf16", True),     # three k-tiles; exactly one CTA of rows and one tile of columns
+    (129, 256, 97, 32, "f32", True),        # one row into the pair's second CTA, one column past its first half of B
+    (257, 1280, 200, 256, "f16", True),     # one row into a second pair tile
+    (60, 4096, 388, 64, "bf16", True),      # 64 offset blocks: past the staging limit; N % 8 != 0: direct stores
+    (33, 1536, 584, 32, "bf16", True),      # 48 offset blocks: the staging limit
+    (520, 512, 15000, 512, "bf16", False),  # more tiles than pairs: both accumulators, a ragged last column tile
+])
+def test_mx_gemm_tile_edges(T, K, N, g, out_dt, rotate):
+    """The block-scaled GEMM at the edges of its tiles, stages, offset staging and output paths."""
+    ldo_ok = N % 8 == 0 or out_dt == "f32" and N % 4 == 0
+    if ldo_ok:
+        _check_mx_layer(T, K, N, g, out_dt, rotate, seed=T + K + N)
+        return
+    # Rows of a wider buffer: a leading dimension that keeps 16-byte alignment.
+    x = W.activations(T, K, seed=T, n_out=3, mult=90.0)
+    w = torch.from_numpy(W.weights(N, K, seed=N)).cuda()
+    ac, ash, asc, aoff = Q.quantize_act_mx(torch.from_numpy(x).to(torch.bfloat16).cuda(), g, rotate=rotate)
+    wide = (N + 7) // 8 * 8
+    outs = []
+    for n in (N, wide):
+        wc, wsh, wsc, wsum = Q.prepare_weight_mx(torch.nn.functional.pad(w, (0, 0, 0, n - N)), g, rotate=rotate)
+        out = torch.zeros((T, wide), dtype=OUT_DT[out_dt], device="cuda")
+        Q.offq_mx_linear(ac, ash, asc, aoff, T, n, K, g, wc, wsh, wsc, wsum, out, wide)
+        outs.append(out[:, :N].clone())
+        if n == N:
+            assert not out[:, N:].any()
+    torch.cuda.synchronize()
+    assert Q.offq_get_device_status() == Q.OFFQ_OK
+    assert torch.equal(outs[0], outs[1])
