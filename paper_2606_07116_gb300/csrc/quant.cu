@@ -976,8 +976,22 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
 // barrier), X kept within 6 of it, then the codes by the E2M1 conversion
 // instruction (round to nearest even, saturating at 6; a code of magnitude 0
 // keeps sign 0), one 16-byte store of the block's codes and its shift byte.
-// With the rotation the values are 32 r (unnormalised by sqrt(1024) = 2^5,
-// exact), so their exponents are offset by 5.
+// With the rotation over g = 1024 the values are 32 r (unnormalised by
+// sqrt(1024) = 2^5, exact), so their exponents are offset by 5.
+//
+// kGen: any offset block and ragged rows. Blocks below 1024 lie within a span
+// (`sub` groups of 32 channels each): the first pass runs the stages of channel
+// bits 5 .. log2 g - 1 only, and block means reduce over the block's lanes;
+// rotations over 2048 .. 8192 exchange the remaining bits between the warps of a
+// block through their scratch; the last span may be short (a multiple of 128).
+// Values are normalised (sqrt(g) need not be a power of two). Bound by latency at
+// few rows and by the per-lane arithmetic at many. One CTA per row with a
+// barrier and two integer divisions per butterfly took, against this form:
+// 1 x 4096 (no rotation) 17.2 us against 2.0, 64 x 11008 (g = 256, rotated) 24.4
+// against 5.5, 2048 x 11008 159 against 42.5, 1000 x 8192 fp32 (g = 8192) 81.9
+// against 25.3. The whole-span instantiation keeps prefill widths (4096 x 14336,
+// g = 1024: 52.8 us either way before; the general one adds the normalisation and
+// the runtime stages to every span).
 
 // floor(log2(a)) for a normal positive fp32 a, from its exponent field.
 __device__ __forceinline__ int floor_log2(float a) { return static_cast<int>((__float_as_uint(a) >> 23) & 0xFF) - 127; }
@@ -999,18 +1013,21 @@ __device__ __forceinline__ uint32_t e2m1_clear_neg_zero(uint32_t w) {
   return mag | (w & nonzero);
 }
 
-template <typename Tin, bool kRot>
+template <typename Tin, bool kRot, bool kGen>
 __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(const QuantArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int abort_flag;
   __shared__ float wpart[k1kMaxWarps];  // per-warp block sums (no rotation, g > 1024)
   __shared__ int wmaxx[k1kMaxWarps];    // per-warp largest block exponent (+ 1024)
   const int K = a.K, R = a.rows_per_cta;
-  const int nbw = K / 1024;  // warps per row
+  const int nbw = kGen ? (K + 1023) / 1024 : K / 1024;  // warps per row
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lrow = warp / nbw;
   const int b = warp - lrow * nbw;          // 1024-channel span of this warp
-  const int m = a.g / 1024;                 // warps per offset block (no rotation)
+  const int m = kGen && a.g < 1024 ? 1 : a.g / 1024;  // warps per offset block
+  const int span = kGen && K - 1024 * b < 1024 ? K - 1024 * b : 1024;  // channels of this warp's span (a multiple of 128)
+  const bool lane_in = !kGen || 32 * lane < span;                     // this lane's MX block exists
+  const int sub = kGen && a.g < 1024 ? a.g / 32 : 32;                 // 32-channel groups per offset block of the span
   const int G = a.G;
   const bool offs = (a.flags & OFFQ_OFFSET) != 0;
   const uint32_t scr32 = smem_u32(smem) + 4096u * warp;  // the warp's transpose scratch (rotation)
@@ -1045,16 +1062,52 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
       if (ok && row_ok) {
         const Tin* p = reinterpret_cast<const Tin*>(ring.slot()) + static_cast<size_t>(lrow) * K + b * 1024 + lane;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = make_float2(smem_elem(p + 64 * i), smem_elem(p + 64 * i + 32));
+        for (int i = 0; i < 16; ++i)
+          v[i] = !kGen || 64 * i < span ? make_float2(smem_elem(p + 64 * i), smem_elem(p + 64 * i + 32))
+                                        : make_float2(0.f, 0.f);
       } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = make_float2(0.f, 0.f);
       }
-      if (offs && lane == 0) {
-        off = v[0].x;
-        v[0].x = 0.f;
+      if constexpr (!kGen) {
+        if (offs && lane == 0) {
+          off = v[0].x;
+          v[0].x = 0.f;
+        }
+        fwht1k_pass(v);  // channel bits 5..9
+      } else {
+        // Every sub-th group of 32 channels (and, for g > 1024, only every m-th warp) starts an offset block.
+        if (lane == 0 && b % m == 0) {
+          float* o = a.offset != nullptr && ok && row_ok
+                         ? a.offset + static_cast<int64_t>(row) * G + (a.g < 1024 ? b * (32 / sub) : b / m)
+                         : nullptr;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            if ((j & (sub - 1)) == 0 && 32 * j < span) {
+              float& x0 = j & 1 ? v[j >> 1].y : v[j >> 1].x;
+              if (o != nullptr) o[j / sub] = offs ? x0 * a.inv_sqrt_g : 0.f;
+              if (offs) x0 = 0.f;
+            }
+          }
+        }
+        if (sub > 1) fwht1k_stage<0>(v);  // channel bits 5 .. log2 g - 1
+        if (sub > 2) fwht1k_stage<1>(v);
+        if (sub > 4) fwht1k_stage<2>(v);
+        if (sub > 8) fwht1k_stage<3>(v);
+        if (sub > 16) fwht1k_stage<4>(v);
+        for (int h = 1; h < m; h <<= 1) {
+          // Channel bits 10 and up: with the partner warp's values, through the scratch.
+          float2* mine = reinterpret_cast<float2*>(smem + 4096 * warp) + lane;
+          const float2* other = reinterpret_cast<const float2*>(smem + 4096 * (warp - b + (b ^ h))) + lane;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) mine[32 * i] = v[i];
+          __syncthreads();
+          const float2 sg = (b & h) != 0 ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(v[i], sg, other[32 * i]);
+          __syncthreads();
+        }
       }
-      fwht1k_pass(v);  // channel bits 5..9
       {
         uint32_t wb[8];
 #pragma unroll
@@ -1077,8 +1130,13 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
         }
       }
       fwht1k_pass(v);  // channel bits 0..4
+      if constexpr (kGen) {
+        const float2 n2 = make_float2(a.inv_sqrt_g, a.inv_sqrt_g);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __fmul2_rn(v[i], n2);
+      }
     } else {
-      if (ok && row_ok) {
+      if (ok && row_ok && lane_in) {
         const Tin* p = reinterpret_cast<const Tin*>(ring.slot()) + static_cast<size_t>(lrow) * K + b * 1024 + 32 * lane;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -1104,7 +1162,10 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
         t8[0] = __fadd2_rn(t8[0], t8[1]);
         float sum = t8[0].x + t8[0].y;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        for (int o = 16; o > 0; o >>= 1) {
+          const float other = __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+          if (!kGen || o < sub) sum += other;  // the lanes of this lane's offset block
+        }
         if (m > 1) {
           if (lane == 0) wpart[warp] = sum;
           __syncthreads();
@@ -1132,7 +1193,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
       mx1 = fmax3(mx1, fabsf(v[i + 1].x), fabsf(v[i + 1].y));
     }
     const float amax = fmaxf(mx0, mx1);
-    constexpr int kUnnorm = kRot ? 5 : 0;  // values are 2^5 r with the rotation
+    constexpr int kUnnorm = kRot && !kGen ? 5 : 0;  // values are 2^5 r with the rotation over g = 1024
     const int xl = amax > 0.f ? floor_log2(amax) - 2 - kUnnorm : -1000;
     const uint32_t wx = __reduce_max_sync(0xFFFFFFFFu, static_cast<uint32_t>(xl + 1024));
     if (lane == 0) wmaxx[warp] = static_cast<int>(wx);
@@ -1159,14 +1220,17 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
       }
       wd[w] = e2m1_clear_neg_zero(bytes[0] | (bytes[1] << 8) | (bytes[2] << 16) | (bytes[3] << 24));
     }
-    if (row_ok) {
+    if (row_ok && lane_in) {
       const int mb = b * 32 + lane;  // the row's MX block
       uint8_t* rdst = a.codes + static_cast<int64_t>(row >> 5) * cpr * 512 + (row & 31) * 16;
       *reinterpret_cast<uint4*>(rdst + static_cast<int64_t>(mb) * 512) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
       a.shifts[((static_cast<int64_t>(row >> 5) * nkt + (mb >> 2)) * 32 + (row & 31)) * 4 + (mb & 3)] =
           static_cast<uint8_t>(X - xlo);
       if (b == 0 && lane == 0) a.scale[row] = pow2f(xlo);
-      if (lane == 0 && a.offset != nullptr) {
+      if (kGen && !kRot && a.g < 1024) {
+        if (a.offset != nullptr && (lane & (sub - 1)) == 0)
+          a.offset[static_cast<int64_t>(row) * G + b * (32 / sub) + lane / sub] = offs ? off : 0.f;
+      } else if (lane == 0 && a.offset != nullptr && !(kGen && kRot)) {
         if constexpr (kRot) {
           a.offset[static_cast<int64_t>(row) * G + b] = offs ? off * 0.03125f : 0.f;
         } else {
@@ -1752,17 +1816,16 @@ int launch_1k(QuantArgs a, cudaStream_t stream) {
 // quantize_mx_1k_kernel: one row of K/1024 warps per CTA (rows per CTA grow
 // while a CTA has fewer than 4 warps), the ring as launch_1k's. kNoRing when the
 // shape does not fit it (the generic MX kernel serves those).
-template <typename Tin, bool kRot>
+template <typename Tin, bool kRot, bool kGen>
 int launch_mx_1k(QuantArgs a, cudaStream_t stream) {
-  const int nbw = a.K / 1024;
-  if (a.H != 1 || a.K % 1024 != 0 || nbw > k1kMaxWarps) return kNoRing;
-  if (kRot ? a.g != 1024 : (a.g % 1024 != 0 || a.g / 1024 > 8)) return kNoRing;
+  const int nbw = (a.K + 1023) / 1024;
+  if (a.H != 1 || nbw > k1kMaxWarps) return kNoRing;
   const int sms = sm_count();
   if (sms <= 0) return OFFQ_ERR_CUDA;
   const int R = std::max(1, 4 / nbw);
   const int64_t groups = (a.rows + R - 1) / R;
-  if (groups <= sms || a.rows + R > 0x7FFFFFFF) return kNoRing;
-  auto kern = quantize_mx_1k_kernel<Tin, kRot>;
+  if (a.rows + R > 0x7FFFFFFF) return kNoRing;
+  auto kern = quantize_mx_1k_kernel<Tin, kRot, kGen>;
   if (prefer_max_shared(kern) != OFFQ_OK) return OFFQ_ERR_CUDA;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxDynSmem)) !=
       cudaSuccess)
@@ -1970,6 +2033,12 @@ __global__ void __launch_bounds__(kRepackWarps * 32) weight_repack_kernel(uint8_
   }
 }
 
+template <typename Tin>
+int launch_mx_rows(const QuantArgs& a, bool rot, bool whole, cudaStream_t s) {
+  if (whole) return rot ? launch_mx_1k<Tin, true, false>(a, s) : launch_mx_1k<Tin, false, false>(a, s);
+  return rot ? launch_mx_1k<Tin, true, true>(a, s) : launch_mx_1k<Tin, false, true>(a, s);
+}
+
 }  // namespace
 
 namespace offq {
@@ -1996,11 +2065,15 @@ int quantize_mx_rows_fast(const void* x, int dtype, int64_t rows, int64_t K, int
   a.shifts = shifts;
   a.g = g;
   const bool rot = (flags & OFFQ_ROTATE) != 0;
+  a.inv_sqrt_g = rot ? static_cast<float>(1.0 / std::sqrt(static_cast<double>(g))) : 1.0f;
+  // Whole spans of 1024 channels with offset blocks of whole spans (g = 1024 with the rotation) have their own
+  // instantiation; blocks within a span, rotations over several and ragged rows take the general one.
+  const bool whole = K % 1024 == 0 && (rot ? g == 1024 : g >= 1024);
   int st = kNoRing;
   switch (dtype) {
-    case OFFQ_BF16: st = rot ? launch_mx_1k<__nv_bfloat16, true>(a, s) : launch_mx_1k<__nv_bfloat16, false>(a, s); break;
-    case OFFQ_F16: st = rot ? launch_mx_1k<__half, true>(a, s) : launch_mx_1k<__half, false>(a, s); break;
-    case OFFQ_F32: st = rot ? launch_mx_1k<float, true>(a, s) : launch_mx_1k<float, false>(a, s); break;
+    case OFFQ_BF16: st = launch_mx_rows<__nv_bfloat16>(a, rot, whole, s); break;
+    case OFFQ_F16: st = launch_mx_rows<__half>(a, rot, whole, s); break;
+    case OFFQ_F32: st = launch_mx_rows<float>(a, rot, whole, s); break;
     default: return OFFQ_ERR_INVALID_ARG;
   }
   return st == kNoRing ? 1 : st;

@@ -16,8 +16,8 @@
 // One CTA per row, the row staged as fp32 in shared memory: the Sylvester
 // transform runs as log2(g) in-place butterfly stages; then a warp per 32-channel
 // block finds the block's exponent, and after the row's maximum is known, its
-// codes. This form serves the format's correctness and the GEMM's inputs; it is
-// not bandwidth-tuned like the per-token quantizer.
+// codes. This form serves weights (offline) and rows of more than 28672 channels;
+// activation rows up to that width take the span form of quant.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -273,8 +273,7 @@ extern "C" int offq_quantize_act_mx(const void* x, int x_dtype, int64_t T, int64
                                     int32_t flags, uint8_t* codes, uint8_t* shifts, float* row_scale, float* offset,
                                     void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // Prefill-sized inputs of 1024-multiple widths take the persistent form; the
-  // arguments are checked by run_mx's rules first (a dry check with zero rows).
+  // Rows of up to 28 spans of 1024 channels take the span form; the arguments are checked by run_mx's rules first (a dry check with zero rows).
   const int chk = run_mx(x, x_dtype, 0, K, ldx, g, flags, codes, shifts, row_scale, offset, nullptr, false, s);
   if (chk != OFFQ_OK) return chk;
   if (T > 0 && x != nullptr && codes != nullptr && shifts != nullptr && row_scale != nullptr &&

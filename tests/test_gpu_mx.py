@@ -212,3 +212,31 @@ def test_mx_gemm_tile_edges(T, K, N, g, out_dt, rotate):
     torch.cuda.synchronize()
     assert Q.offq_get_device_status() == Q.OFFQ_OK
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("T,K,g,rotate,dt", [
+    (3, 128, 32, True, "bf16"),       # one ragged span of four lanes; no stage above bit 4
+    (5, 1152, 128, True, "f16"),      # a whole span and a ragged one
+    (4, 1152, 128, False, "f32"),     # the same, block means over 4 lanes
+    (9, 11008, 256, False, "bf16"),   # 11 spans, the last of 768 channels
+    (2, 2048, 2048, True, "bf16"),    # rotation over two warps (two rows per CTA)
+    (3, 8192, 8192, True, "f32"),     # over eight
+    (6, 3072, 512, True, "bf16"),
+    (1, 4096, 1024, True, "bf16"),    # the whole-span form at one row
+    (40, 28672, 4096, True, "bf16"),  # 28 warps, rotations over four
+])
+def test_mx_quantizer_spans(T, K, g, rotate, dt):
+    """The span form over block widths within a span, over several spans and with ragged last spans; without
+    offsets, the codes' zero-offset rows too."""
+    x = W.activations(T, K, seed=T + K + g, n_out=2, mult=60.0)
+    xe, codes, shifts, scale, off = _quant(x, g, rotate, dt)
+    ref = O.quantize_act_mx(xe, g, rotate=rotate, offset=True)
+    code, sh, X = _decode(codes, shifts, scale, T, K)
+    check_mx(code, X, ref, xe, g, rotate)
+    check_offsets(off.cpu().numpy(), ref["offset"], xe, g, rotate)
+    xt = torch.from_numpy(x).to(OUT_DT[dt] if dt != "f32" else torch.float32).cuda()
+    codes, shifts, scale, off = Q.quantize_act_mx(xt, g, rotate=rotate, offset=False)
+    ref = O.quantize_act_mx(xe, g, rotate=rotate, offset=False)
+    code, sh, X = _decode(codes, shifts, scale, T, K)
+    check_mx(code, X, ref, xe, g, rotate)
+    assert not off.any()
