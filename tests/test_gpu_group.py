@@ -191,9 +191,8 @@ def test_group_gemm_is_repeatable():
 
 
 def test_group_gemm_zero_points_outside_the_code_range():
-    """Groups that do not straddle zero have z = -rne(min/s) outside [0, 15]:
-    the kernel subtracts clamp(z, 0, 15) in the operand and the rest through
-    the weight group sums. Shifted groups are mixed with ordinary ones within
+    """Groups that do not straddle zero have z = -rne(min/s) outside [0, 15];
+    the kernel subtracts z times the weight group sums. Shifted groups are mixed with ordinary ones within
     each warp's 32 rows."""
     T, K, N = 300, 1024, 640
     x = W.activations(T, K, seed=90, n_out=3, mult=60.0)
@@ -209,3 +208,15 @@ def test_group_gemm_zero_points_outside_the_code_range():
     z = zero.cpu().numpy()
     assert (z < 0).any() and (z > 15).any() and ((z >= 0) & (z <= 15)).any()
     _check_group_layer(T, K, N, 1024, "f32", False, x=x)
+
+
+@pytest.mark.parametrize("T,K,N,out_dt", [
+    (1, 128, 8, "f32"),        # one group: a window of one, one row, a few columns
+    (33, 2048, 129, "f16"),    # exactly one window of 16 groups; one column past a tile; N % 4 != 0 (scalar copies of R)
+    (129, 2176, 64, "bf16"),   # 17 groups: a second window of one; rows of s and z not a multiple of 16 bytes
+    (257, 640, 100, "f32"),    # 5 groups, one row into a second pair tile
+    (64, 4608, 520, "bf16"),   # 36 groups: three windows, the last of four
+])
+def test_group_gemm_windows(T, K, N, out_dt):
+    """The group GEMM at the edges of its windows of s, z and R, its tiles and their copies' alignment."""
+    _check_group_layer(T, K, N, 128, out_dt, False, seed=T + K, ldo=(N + 7) // 8 * 8)
