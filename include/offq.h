@@ -181,10 +181,11 @@ int offq_quantize_act(const void* x, int x_dtype, int64_t T, int64_t K, int64_t 
  *   acc_debug device, [T][N] int32 or NULL. When given, also receives the
  *             integer the tensor cores accumulate, sum_k (q_a + 8) * q_w
  *             (equal to the true dot product plus 8 * sum_k q_w[n][k]).
- * Forms: T > 64 the pair-tile tensor-core kernel; 33 <= T <= 64 the decode
- * kernel (weights on the MMA's M side); T <= 32 the few-token form (weights
- * straight into registers, warp-level MMA). All give the same accumulator and
- * apply the same epilogue.
+ * Forms: T <= 32 the few-token form (weights straight into registers,
+ * warp-level MMA); above, the pair-tile tensor-core kernel, or, where its 256 x
+ * 256 tiles are too few to fill the chip, the form that gives a CTA 128 output
+ * channels x up to 128 tokens and splits K over a cluster. All give the same
+ * accumulator and apply the same epilogue.
  * Ordering: the T <= 32 form starts reading w_codes, w_scale and w_offsum
  * before the kernel ahead of it in the stream has finished (programmatic
  * dependent launch), so they must not be written by a kernel that releases its

@@ -158,6 +158,22 @@ def test_few_token_form(T, K, N, g, out_dt):
     _check_layer(T, K, N, g, out_dt, ldo=ldo, seed=T * 7 + K)
 
 
+@pytest.mark.parametrize("T,K,N,g,out_dt", [
+    (33, 128, 40, 128, "f32"),       # one k-tile, 48 token columns, no split of K
+    (40, 1056, 129, 32, "bf16"),     # a short last k-tile; one channel into a second tile; 33 offset blocks
+    (65, 8192, 1000, 8192, "f16"),   # K over eight CTAs, 80 token columns (five chunks: three CTAs own none)
+    (128, 4096, 264, 4096, "bf16"),  # a whole token tile, K over eight
+    (129, 4096, 1024, 1024, "f32"),  # two token tiles of 80: the second starts inside a 32-row block
+    (200, 2048, 4096, 32, "bf16"),   # 64 offset blocks
+    (70, 4096, 512, 32, "f32"),      # 128 offset blocks: read from global memory
+    (300, 11008, 4096, 256, "bf16"), # three token tiles of 112
+    (48, 512, 8200, 512, "f16"),     # short K: no split; a ragged last channel tile
+])
+def test_mid_form(T, K, N, g, out_dt):
+    """The form between decode and prefill at the edges of its tiles, K splits and offset staging."""
+    _check_layer(T, K, N, g, out_dt, ldo=(N + 7) // 8 * 8, seed=T + K)
+
+
 def test_no_rotation_site():
     """q/k/v/gate/up sites: codes made without the online rotation."""
     _check_layer(64, 4096, 768, 4096, "bf16", rotate=False, seed=5)
@@ -337,7 +353,7 @@ def test_outputs_near_zero_against_large_row_sums(K, g):
 
 
 def test_few_token_forms_agree():
-    """4 tokens take the CUDA-core form, 5 to 9 the tensor-core decode kernel: on the same rows
+    """4 to 8 tokens take the one-tile few-token form, 9 the two-tile one: on the same rows
     both give the same integer accumulators and, with the same epilogue chain, the same
     output bits."""
     T, K, N, g = 9, 4096, 11008, 4096
