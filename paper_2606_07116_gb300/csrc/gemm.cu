@@ -59,7 +59,7 @@ constexpr int BK = 128;            // codes per k-tile
 constexpr int kChunksPerKt = BK / 32;  // 16-byte packed chunks per row per k-tile
 // Warp roles of one instantiation. kSplitA / kSplitB converter warps serve each
 // 32-row group of A / B, taking turns by k-tile; kEpiWarps drain the
-// accumulator (one or two per 32-lane TMEM quarter). 21 warps put 6 on one SM
+// accumulator (one per 32-lane TMEM quarter). 21 warps put 6 on one SM
 // sub-partition: 80 registers per thread. (Trading B converters for epilogue
 // warps in the several-block kernel left one B warp per group too slow.)
 template <bool kOneBlock>
@@ -70,8 +70,7 @@ struct Roles {
   static constexpr int kSplitA = 2;
   static constexpr int kSplitB = 2;
   static constexpr int kAWarps = 4 * kSplitA, kBWarps = 4 * kSplitB;
-  static constexpr int kEpiWarps = 4;
-  static constexpr int kEpiCols = BN / (kEpiWarps / 4);  // accumulator columns per epilogue warp
+  static constexpr int kEpiWarps = 4;  // one per 32-lane TMEM quarter
   static constexpr int kFirstA = 1, kFirstB = kFirstA + kAWarps, kFirstEpi = kFirstB + kBWarps;
   static constexpr int kThreads = (kFirstEpi + kEpiWarps) * 32;
   static_assert(kSplitA <= kStages && kSplitB <= kStages, "a converter's next stage is at most one ring turn ahead");
@@ -94,31 +93,31 @@ static_assert(kACol0 + Roles<true>::kStages * kAColsPerStage <= kTmemCols, "TMEM
 constexpr int kCorrCol0 = kACol0 + Roles<false>::kStages * kAColsPerStage;
 constexpr int kCorrTmemCols = 128;
 static_assert(kCorrCol0 + kCorrTmemCols <= kTmemCols, "TMEM budget with the correction");
-constexpr int kCorrPitch = (BN - kCorrTmemCols) * 4 + 16;  // bytes per row of the shared half, padded
-
 constexpr int kBStage = BNH * BK;  // 16 KB of E4M3 per stage
-// Output rows staged by the one-block epilogue (16-bit outputs): pitch padded
-// by 16 bytes, so the 32 rows a warp writes at once fall in distinct bank groups.
+// Output rows staged by the epilogue (16-bit outputs): pitch padded by 16
+// bytes, so the 32 rows a warp writes at once fall in distinct bank groups. The
+// correction's columns 128..255 lie in the same bytes of their row before.
 constexpr int kOutPitch = BN * 2 + 16;
+static_assert((BN - kCorrTmemCols) * 4 + 16 == kOutPitch, "a row's correction half and its outputs share the buffer");
 
 // Shared memory of one instantiation: B stages; the tile's epilogue constants
-// (row sums R[b][256 columns], channel scales, per row o[t][b] - 8 s_a[t] with
-// an odd pitch for conflict-free per-lane reads, s_a); for one offset block the
-// staged output rows; barriers.
+// (row sums R[b][256 columns], channel scales, offsets o[b][128 rows], s_a);
+// the staged output rows, which several offset blocks share with half of their
+// correction; barriers.
 template <bool kOneBlock>
 struct Smem {
   static constexpr int kStages = Roles<kOneBlock>::kStages;
   static constexpr int kNumBars = 2 * kStages + 2;
   static constexpr int kMaxG = kOneBlock ? 1 : kMaxStageG;
-  static constexpr int kGp = kOneBlock ? 1 : kMaxStageG + 1;
+  static constexpr int kOPitch = kOneBlock ? BM : BM + 4;  // floats per block of staged offsets
   static constexpr int kOffB = 0;
   static constexpr int kOffR = kOffB + kStages * kBStage;
   static constexpr int kOffW = kOffR + kMaxG * BN * 4;
   static constexpr int kOffO = kOffW + BN * 4;
-  static constexpr int kOffSa = kOffO + BM * kGp * 4;
-  static constexpr int kOffRt = kOffSa + BM * 4;    // several blocks: -8 Rt[n] 2^-18 per column
-  static constexpr int kOffOut = kOffRt + BN * 4;   // one block: staged output rows; several: the correction half
-  static constexpr int kOffBars = kOffOut + (kOneBlock ? BM * kOutPitch : BM * kCorrPitch);
+  static constexpr int kOffSa = kOffO + kMaxG * kOPitch * 4;
+  static constexpr int kOffRt = kOffSa + BM * 4;    // several blocks: -8 sum_b R[b][n] per column
+  static constexpr int kOffOut = kOffRt + BN * 4;   // staged output rows; several blocks: first the correction half
+  static constexpr int kOffBars = kOffOut + BM * kOutPitch;
   static constexpr int kOffMisc = kOffBars + kNumBars * 8;
   static constexpr int kBytes = kOffMisc + 64 + 1024;  // + slack to align the base to 1024
   static_assert(kBytes <= 227 * 1024, "shared memory budget");
@@ -144,7 +143,7 @@ struct GemmParams {
   int t_blocks, n_blocks;  // 32-row tiles present in the code buffers
   int kchunks;             // K / 32
   int vec_ok;              // rowsum and w_scale rows are 16-byte aligned
-  int async_out;           // 16-bit output and N % 8 == 0: one-block rows leave by bulk copy
+  int async_out;           // 16-bit output, N % 8 == 0, no debug output: rows leave by bulk copy
 };
 
 // Loads the four 16-byte chunks of k-tile kt of one row of a tiled code matrix
@@ -179,6 +178,56 @@ __device__ __forceinline__ void tile_mn(const GemmParams& p, int tile, int& mp, 
   mp = grp * p.raster_m + (local - nt * gm);
 }
 
+// Waits for the TMEM loads into r; the statement also hands the registers on, so
+// nothing reads them before it.
+__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_8cols(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+// 16 TMEM lanes x 32 columns: lane l of the warp gives, for each 8-column group
+// j, row l / 4 columns 2 (l % 4) and + 1 in r[4j], r[4j + 1] and row l / 4 + 8 in
+// r[4j + 2], r[4j + 3].
+__device__ __forceinline__ void tmem_st_16rows_32cols(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+template <int kBytes>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(kBytes) : "memory");
+}
+template <int OUT>
+__device__ __forceinline__ uint32_t pack_out(float a, float b) {
+  if (OUT == OFFQ_BF16) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  const __half2 v = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // Row block (of 32 rows) of this CTA's A rows / B rows for a pair tile.
 __device__ __forceinline__ int a_block(const GemmParams& p, int tile, uint32_t rank, int quarter) {
   int mp, nt;
@@ -209,9 +258,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
   using RL = Roles<kOneBlock>;
   constexpr int kStages = RL::kStages;
   constexpr int kFirstA = RL::kFirstA, kFirstB = RL::kFirstB, kFirstEpi = RL::kFirstEpi;
-  constexpr int kEpiWarps = RL::kEpiWarps, kEpiCols = RL::kEpiCols;
+  constexpr int kEpiWarps = RL::kEpiWarps;
   constexpr int kOffB = SL::kOffB, kOffR = SL::kOffR, kOffW = SL::kOffW, kOffO = SL::kOffO, kOffSa = SL::kOffSa;
-  constexpr int kOffBars = SL::kOffBars, kOffMisc = SL::kOffMisc, kStageGp = SL::kGp;
+  constexpr int kOffBars = SL::kOffBars, kOffMisc = SL::kOffMisc, kOPitch = SL::kOPitch;
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - raw);
@@ -400,7 +449,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
     // ---------------- epilogue ----------------
     const uint64_t out_pol = l2_evict_first();  // outputs: nothing here reads them again
     const int quarter = warp & 3;              // TMEM lanes this warp may read
-    const int half = (warp - kFirstEpi) / 4;   // which kEpiCols accumulator columns
     const int et = threadIdx.x - kFirstEpi * 32;
     const int G = kOneBlock ? 1 : p.G;
     // More offset blocks than the staging area holds take their own
@@ -410,10 +458,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
     float* Ws = reinterpret_cast<float*>(smem + kOffW);
     float* Os = reinterpret_cast<float*>(smem + kOffO);
     float* Sa = reinterpret_cast<float*>(smem + kOffSa);
-    float* Rt = reinterpret_cast<float*>(smem + SL::kOffRt);
+    float* Rt = reinterpret_cast<float*>(smem + SL::kOffRt);  // several blocks: -8 sum_b R[b][n]
     const uint32_t acc_empty_l = leader_addr(acc_empty);
     // Loop exit decided only from a flag the epilogue warps write before their
-    // own barrier, so all eight warps leave together (bar.sync has no timeout).
+    // own barrier, so all its warps leave together (bar.sync has no timeout).
     volatile int* epi_stop = reinterpret_cast<volatile int*>(smem + kOffMisc + 32);
     if (et == 0) *epi_stop = 0;
     epi_sync<kEpiWarps>();
@@ -424,78 +472,131 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
       const int m0 = mp * 2 * BM + static_cast<int>(rank) * BM;
       const int nt0 = nt * BN;
       // Stage this tile's constants while the main loop runs.
-      if (staged) {
-        for (int i = et; i < G * BN; i += kEpiWarps * 32) {
-          const int b = i / BN, j = i - b * BN, n = nt0 + j;
-          Rs[i] = n < p.N ? __ldg(p.rowsum + static_cast<int64_t>(b) * p.N + n) : 0.f;
-        }
-        for (int i = et; i < BN; i += kEpiWarps * 32) Ws[i] = nt0 + i < p.N ? __ldg(p.w_scale + nt0 + i) : 0.f;
-        for (int i = et; i < BM; i += kEpiWarps * 32) Sa[i] = m0 + i < p.T ? __ldg(p.a_scale + m0 + i) : 0.f;
-        for (int i = et; i < BM * G; i += kEpiWarps * 32) {
-          const int r = i / G, b = i - r * G, t = m0 + r;
-          float v = 0.f;
-          if (t < p.T && p.a_offset != nullptr) v = __ldg(p.a_offset + static_cast<int64_t>(t) * G + b);
-          Os[r * kStageGp + b] = v;
-        }
-      }
-      epi_sync<kEpiWarps>();
-      if (!kOneBlock && staged) {
-        // Rt[n] * 8 * 2^-18 = sum_b R[b][n] * 2^-15: integers, exact in fp32.
+      if constexpr (kOneBlock) {
         for (int i = et; i < BN; i += kEpiWarps * 32) {
-          float r = 0.f;
-          for (int b = 0; b < G; ++b) r += Rs[b * BN + i];
-          Rt[i] = r * -0x1p-15f;
+          const bool in = nt0 + i < p.N;
+          Rs[i] = in ? __ldg(p.rowsum + nt0 + i) : 0.f;
+          Ws[i] = in ? __ldg(p.w_scale + nt0 + i) : 0.f;
         }
+        const bool in = m0 + et < p.T;
+        Sa[et] = in ? __ldg(p.a_scale + m0 + et) : 0.f;
+        Os[et] = in && p.a_offset != nullptr ? __ldg(p.a_offset + m0 + et) : 0.f;
         epi_sync<kEpiWarps>();
-      }
-      if constexpr (!kOneBlock) {
-        if (staged) {
-          // While this tile's MMAs run: its offset correction, per element the same
-          // chain as at the tile end (block 0 multiplied, then FMAs in block order).
-          constexpr int CW = 16;
-          const int rl = quarter * 32 + lane;
-          const float* orow = Os + rl * kStageGp;
-          const uint32_t corr_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kCorrCol0;
-          const uint32_t corr_s = base + SL::kOffOut + rl * kCorrPitch;
-          for (int c = 0; c < kEpiCols / CW; ++c) {
-            const int jc = half * kEpiCols + c * CW;  // column within the tile
-            float y[CW];
-            {
-              const float ob = orow[0];
-              const float4* r4 = reinterpret_cast<const float4*>(Rs + jc);
-#pragma unroll
-              for (int q4 = 0; q4 < CW / 4; ++q4) {
-                const float4 rv = r4[q4];
-                y[4 * q4] = ob * rv.x; y[4 * q4 + 1] = ob * rv.y; y[4 * q4 + 2] = ob * rv.z; y[4 * q4 + 3] = ob * rv.w;
-              }
-            }
-            for (int b = 1; b < G; ++b) {
-              const float ob = orow[b];
-              const float4* r4 = reinterpret_cast<const float4*>(Rs + b * BN + jc);
-#pragma unroll
-              for (int q4 = 0; q4 < CW / 4; ++q4) {
-                const float4 rv = r4[q4];
-                y[4 * q4] = fmaf(ob, rv.x, y[4 * q4]);
-                y[4 * q4 + 1] = fmaf(ob, rv.y, y[4 * q4 + 1]);
-                y[4 * q4 + 2] = fmaf(ob, rv.z, y[4 * q4 + 2]);
-                y[4 * q4 + 3] = fmaf(ob, rv.w, y[4 * q4 + 3]);
-              }
-            }
-            if (jc < kCorrTmemCols) {
-              uint32_t u[CW];
-#pragma unroll
-              for (int jj = 0; jj < CW; ++jj) u[jj] = __float_as_uint(y[jj]);
-              tmem_st_16cols(corr_tm + jc, u);
-            } else {
-              const uint32_t a = corr_s + (jc - kCorrTmemCols) * 4;
-#pragma unroll
-              for (int q4 = 0; q4 < CW / 4; ++q4)
-                sts128(a + 16 * q4, __float_as_uint(y[4 * q4]), __float_as_uint(y[4 * q4 + 1]),
-                       __float_as_uint(y[4 * q4 + 2]), __float_as_uint(y[4 * q4 + 3]));
-            }
+      } else if constexpr (staged) {
+        // Asynchronous copies, so their latencies overlap: 9.5 k cycles at 43 blocks (22 k as loads into registers).
+        // R: thread et takes columns 2 et and 2 et + 1 of every block, placed so that the 8 columns a lane multiplies
+        // below are 32 contiguous bytes.
+        const int c2 = 2 * et, n2 = nt0 + c2;
+        float* rdst = Rs + (c2 & ~31) + (c2 & 7) * 4 + ((c2 >> 3) & 3) * 2;
+        if (p.vec_ok && n2 < p.N) {
+          const float* src = p.rowsum + n2;
+          for (int b = 0; b < G; ++b, src += p.N) cp_async<8>(smem_u32(rdst + b * BN), src);
+        } else {
+          for (int b = 0; b < G; ++b) {
+            const float* src = p.rowsum + static_cast<int64_t>(b) * p.N + n2;
+            rdst[b * BN] = n2 < p.N ? __ldg(src) : 0.f;
+            rdst[b * BN + 1] = n2 + 1 < p.N ? __ldg(src + 1) : 0.f;
           }
-          tmem_st_wait();
         }
+        Ws[c2] = n2 < p.N ? __ldg(p.w_scale + n2) : 0.f;
+        Ws[c2 + 1] = n2 + 1 < p.N ? __ldg(p.w_scale + n2 + 1) : 0.f;
+        Sa[et] = m0 + et < p.T ? __ldg(p.a_scale + m0 + et) : 0.f;
+        // Offsets, [b][row]: rows q, q + 8, q + 16, q + 24 of a 32-row group side by side.
+        const int64_t left = static_cast<int64_t>(p.T - m0) * G;  // offsets from row m0 on; not positive past the end
+        const float* o0 = p.a_offset + static_cast<int64_t>(m0) * G;
+        const int step_r = kEpiWarps * 32 / G, step_b = kEpiWarps * 32 - step_r * G;
+        int r = et / G, b = et - r * G;
+        for (int i = et; i < BM * G; i += kEpiWarps * 32) {
+          float* dst = Os + b * kOPitch + (r & ~31) + (r & 7) * 4 + ((r >> 3) & 3);
+          if (p.a_offset != nullptr && i < left)
+            cp_async<4>(smem_u32(dst), o0 + i);
+          else
+            *dst = 0.f;
+          r += step_r;
+          b += step_b;
+          if (b >= G) {
+            b -= G;
+            ++r;
+          }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        {
+          // Rt[n] = -8 sum_b R[b][n]: integers, exact in fp32. (This thread's own copies.)
+          float r0 = 0.f, r1 = 0.f;
+#pragma unroll 4
+          for (int bb = 0; bb < G; ++bb) {
+            const float2 v = *reinterpret_cast<const float2*>(rdst + bb * BN);
+            r0 += v.x;
+            r1 += v.y;
+          }
+          Rt[c2] = r0 * -8.f;
+          Rt[c2 + 1] = r1 * -8.f;
+        }
+        if (p.async_out) bulk_wait_read_all();  // this row's previous output copy has read the buffer
+        epi_sync<kEpiWarps>();
+        // While this tile's MMAs run: its offset correction, per element the same chain as at the tile end (block 0
+        // multiplied, then FMAs in block order). A lane takes 4 rows x 8 columns at a time, the fragment that a
+        // 16-lane x 256-bit TMEM store takes: 3 shared reads of 16 bytes per 32 multiply-adds, where one row and 16
+        // columns per lane took 5 per 16. With 43 blocks it still is the longest part of a tile (2048 tokens x 11008 ->
+        // 4096 98.6 -> 74.5 us with the staging and the drain): 59 k cycles, about half of them multiply-adds at one
+        // warp per sub-partition. Reading a block ahead (81 us: registers) and scalar multiply-adds (80 us) were slower.
+        const int q = lane >> 2, m = lane & 3;
+        const float* op = Os + quarter * 32 + q * 4;
+        const uint32_t corr_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kCorrCol0;
+        const uint32_t corr_s = base + SL::kOffOut + (quarter * 32 + q) * kOutPitch + m * 8;
+        for (int sb = 0; sb < BN / 32; ++sb) {
+          const float* rp = Rs + sb * 32 + m * 8;
+          uint64_t y[4][4];  // [row q + 8 i][column pair 8 j + 2 m]
+          {
+            const float4 o = *reinterpret_cast<const float4*>(op);
+            const float4 ra = *reinterpret_cast<const float4*>(rp), rb = *reinterpret_cast<const float4*>(rp + 4);
+            const uint64_t R[4] = {pack2(ra.x, ra.y), pack2(ra.z, ra.w), pack2(rb.x, rb.y), pack2(rb.z, rb.w)};
+            const uint64_t O[4] = {pack2(o.x, o.x), pack2(o.y, o.y), pack2(o.z, o.z), pack2(o.w, o.w)};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) y[i][j] = mul2v(O[i], R[j]);
+          }
+#pragma unroll 2
+          for (int bb = 1; bb < G; ++bb) {
+            const float4 o = *reinterpret_cast<const float4*>(op + bb * kOPitch);
+            const float4 ra = *reinterpret_cast<const float4*>(rp + bb * BN);
+            const float4 rb = *reinterpret_cast<const float4*>(rp + bb * BN + 4);
+            const uint64_t R[4] = {pack2(ra.x, ra.y), pack2(ra.z, ra.w), pack2(rb.x, rb.y), pack2(rb.z, rb.w)};
+            const uint64_t O[4] = {pack2(o.x, o.x), pack2(o.y, o.y), pack2(o.z, o.z), pack2(o.w, o.w)};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) y[i][j] = fma2v(O[i], R[j], y[i][j]);
+          }
+          if (sb * 32 < kCorrTmemCols) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t u[16];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float v0, v1, v2, v3;
+                unpack2(y[2 * h][j], v0, v1);
+                unpack2(y[2 * h + 1][j], v2, v3);
+                u[4 * j] = __float_as_uint(v0); u[4 * j + 1] = __float_as_uint(v1);
+                u[4 * j + 2] = __float_as_uint(v2); u[4 * j + 3] = __float_as_uint(v3);
+              }
+              tmem_st_16rows_32cols(corr_tm + (static_cast<uint32_t>(16 * h) << 16) + sb * 32, u);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float v0, v1;
+                unpack2(y[i][j], v0, v1);
+                sts64(corr_s + 8 * i * kOutPitch + (sb * 32 - kCorrTmemCols + 8 * j) * 4, __float_as_uint(v0),
+                      __float_as_uint(v1));
+              }
+          }
+        }
+        tmem_st_wait();
+        __syncwarp();  // a row's correction comes from four lanes
       }
       const bool ok = __all_sync(0xFFFFFFFFu, wait_cluster(acc_full, lt & 1, abort));
       if (!ok && lane == 0) *epi_stop = 1;
@@ -503,29 +604,168 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
       const int rl = quarter * 32 + lane;
       const int t = m0 + rl;
       const bool row_ok = t < p.T;
-      const int n0 = nt0 + half * kEpiCols;
-      const uint32_t acc_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + half * kEpiCols;
+      const uint32_t acc_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
       constexpr int CW = 16;  // accumulator columns per TMEM load
+      bool released = false;
+      // The accumulator has been read: the next tile's MMAs may start.
+      auto release = [&] {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_cluster(acc_empty_l);
+        released = true;
+      };
+      const uint32_t orow_s = base + SL::kOffOut + rl * kOutPitch;
+      const bool async_out = OUT != OFFQ_F32 && !kUnstaged && p.async_out != 0;
       if (!ok) {
         // Aborted: nothing to drain.
-      } else if (!kOneBlock && staged) {
-        // Several offset blocks: the correction was computed during the main loop.
-        const float sa = Sa[rl];
-        const uint32_t corr_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kCorrCol0;
-        const uint32_t corr_s = base + SL::kOffOut + rl * kCorrPitch;
-        for (int c = 0; c < kEpiCols / CW; ++c) {
-          const int jc = half * kEpiCols + c * CW;  // column within the tile
-          uint32_t acc[CW], cr[CW];
-          tmem_ld_16cols(acc_tm + c * CW, acc);
-          if (jc < kCorrTmemCols) tmem_ld_16cols(corr_tm + jc, cr);
-          tmem_ld_wait();
-          const int nb = n0 + c * CW;
-          if (!row_ok || nb >= p.N) continue;
-          if (jc >= kCorrTmemCols) {
-            const uint32_t a = corr_s + (jc - kCorrTmemCols) * 4;
+      } else if (async_out) {
+        // 16-bit rows go to shared memory and leave by one bulk copy per row, so the tile's output write overlaps the
+        // next tile's MMAs. No MMA runs during the drain, so its length adds to the tile: the next columns are on
+        // their way while these are scaled, and the accumulator is handed back before the last of them and the copies.
+        // Rows and columns past the end are computed from zeros and not copied, so no lane branches. 9.2 k cycles
+        // before, of a tile's 30 k at K = 4096, now 2.9 k: 8192 tokens x 4096 -> 4096 98 -> 89 us, -> 11008 248 ->
+        // 222 us; 14 blocks of 1024 -> 4096 at 2048 tokens (there with strided 32-byte stores) 93 -> 88 us.
+        if constexpr (kOneBlock) {
+          // Packed fp32 pairs; each lane rounds as y = s_w * fma(s_a, acc * 2^18, o R)
+          // does, with acc = (acc' - 8 R) 2^-18 formed exactly first (s_a * 2^18 and
+          // its product with acc are exact).
+          const float sa2 = Sa[rl] * kAccScale;
+          const float ob = Os[rl];
+          const uint64_t SA2 = pack2(sa2, sa2), OB = pack2(ob, ob);
+          const uint64_t M8 = pack2(-0x1p-15f, -0x1p-15f);  // -8 * 2^-18
+          bulk_wait_read_all();  // this row's previous copy has read the buffer
+          auto emit = [&](int c, const uint32_t (&acc)[CW]) {
+            const float4* r4 = reinterpret_cast<const float4*>(Rs + c * CW);
+            const float4* w4 = reinterpret_cast<const float4*>(Ws + c * CW);
+            uint32_t hv[CW / 2];
 #pragma unroll
             for (int q4 = 0; q4 < CW / 4; ++q4) {
-              const uint4 v = lds128(a + 16 * q4);
+              const float4 rv = r4[q4], wv = w4[q4];
+              const uint64_t R0 = pack2(rv.x, rv.y), R1 = pack2(rv.z, rv.w);
+              uint64_t A0 = pack2(__uint_as_float(acc[4 * q4]), __uint_as_float(acc[4 * q4 + 1]));
+              uint64_t A1 = pack2(__uint_as_float(acc[4 * q4 + 2]), __uint_as_float(acc[4 * q4 + 3]));
+              A0 = fma2v(R0, M8, A0);
+              A1 = fma2v(R1, M8, A1);
+              float y0, y1, y2, y3;
+              unpack2(mul2v(pack2(wv.x, wv.y), fma2v(SA2, A0, mul2v(OB, R0))), y0, y1);
+              unpack2(mul2v(pack2(wv.z, wv.w), fma2v(SA2, A1, mul2v(OB, R1))), y2, y3);
+              hv[2 * q4] = pack_out<OUT>(y0, y1);
+              hv[2 * q4 + 1] = pack_out<OUT>(y2, y3);
+            }
+            sts128(orow_s + c * CW * 2, hv[0], hv[1], hv[2], hv[3]);
+            sts128(orow_s + c * CW * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
+          };
+          uint32_t a0[CW], a1[CW];
+          tmem_ld_16cols(acc_tm, a0);
+#pragma unroll
+          for (int c = 0; c < BN / CW; c += 2) {
+            tmem_ld_wait_for(a0);
+            tmem_ld_16cols(acc_tm + (c + 1) * CW, a1);
+            emit(c, a0);
+            tmem_ld_wait_for(a1);
+            if (c + 2 < BN / CW)
+              tmem_ld_16cols(acc_tm + (c + 2) * CW, a0);
+            else
+              release();
+            emit(c + 1, a1);
+          }
+        } else {
+          // Several blocks: columns 128..255 first, from the highest down, because their outputs overwrite corrections
+          // of higher columns of the row; then 0..127, whose corrections are in TMEM.
+          const float sa = Sa[rl];
+          const uint64_t SA = pack2(sa, sa), K18 = pack2(kAccScale, kAccScale);
+          const uint32_t corr_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kCorrCol0;
+          // z = s_w * fma(s_a, acc' 2^18 + Rt, correction) of 4 columns from j; the inner sum is an exact integer.
+          auto four = [&](int j, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint64_t c0, uint64_t c1,
+                          uint32_t& h0, uint32_t& h1) {
+            const float4 rt = *reinterpret_cast<const float4*>(Rt + j), wv = *reinterpret_cast<const float4*>(Ws + j);
+            const uint64_t A0 = fma2v(pack2(__uint_as_float(x0), __uint_as_float(x1)), K18, pack2(rt.x, rt.y));
+            const uint64_t A1 = fma2v(pack2(__uint_as_float(x2), __uint_as_float(x3)), K18, pack2(rt.z, rt.w));
+            float y0, y1, y2, y3;
+            unpack2(mul2v(pack2(wv.x, wv.y), fma2v(SA, A0, c0)), y0, y1);
+            unpack2(mul2v(pack2(wv.z, wv.w), fma2v(SA, A1, c1)), y2, y3);
+            h0 = pack_out<OUT>(y0, y1);
+            h1 = pack_out<OUT>(y2, y3);
+          };
+          auto pair2 = [](uint32_t a, uint32_t b) { return pack2(__uint_as_float(a), __uint_as_float(b)); };
+          auto emit_s = [&](int c, const uint32_t (&acc)[CW]) {
+            uint32_t hv[CW / 2];
+#pragma unroll
+            for (int q4 = 0; q4 < CW / 4; ++q4) {
+              const uint4 v = lds128(orow_s + (c * CW - kCorrTmemCols) * 4 + 16 * q4);
+              four(c * CW + 4 * q4, acc[4 * q4], acc[4 * q4 + 1], acc[4 * q4 + 2], acc[4 * q4 + 3], pair2(v.x, v.y),
+                   pair2(v.z, v.w), hv[2 * q4], hv[2 * q4 + 1]);
+            }
+            sts128(orow_s + c * CW * 2, hv[0], hv[1], hv[2], hv[3]);
+            sts128(orow_s + c * CW * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
+          };
+          {
+            constexpr int kFirst = kCorrTmemCols / CW, kLast = BN / CW - 1;
+            uint32_t a0[CW], a1[CW];
+            tmem_ld_16cols(acc_tm + kLast * CW, a0);
+#pragma unroll
+            for (int c = kLast; c > kFirst; c -= 2) {
+              tmem_ld_wait_for(a0);
+              tmem_ld_16cols(acc_tm + (c - 1) * CW, a1);
+              emit_s(c, a0);
+              tmem_ld_wait_for(a1);
+              if (c - 2 > kFirst) tmem_ld_16cols(acc_tm + (c - 2) * CW, a0);
+              emit_s(c - 1, a1);
+            }
+          }
+          auto emit_t = [&](int j, const uint32_t (&acc)[8], const uint32_t (&cr)[8]) {
+            uint32_t hv[4];
+#pragma unroll
+            for (int q4 = 0; q4 < 2; ++q4)
+              four(j + 4 * q4, acc[4 * q4], acc[4 * q4 + 1], acc[4 * q4 + 2], acc[4 * q4 + 3],
+                   pair2(cr[4 * q4], cr[4 * q4 + 1]), pair2(cr[4 * q4 + 2], cr[4 * q4 + 3]), hv[2 * q4],
+                   hv[2 * q4 + 1]);
+            sts128(orow_s + j * 2, hv[0], hv[1], hv[2], hv[3]);
+          };
+          uint32_t a0[8], c0[8], a1[8], c1[8];
+          tmem_ld_8cols(acc_tm, a0);
+          tmem_ld_8cols(corr_tm, c0);
+#pragma unroll
+          for (int j = 0; j < kCorrTmemCols; j += 16) {
+            tmem_ld_wait_for(a0, c0);
+            tmem_ld_8cols(acc_tm + j + 8, a1);
+            tmem_ld_8cols(corr_tm + j + 8, c1);
+            emit_t(j, a0, c0);
+            tmem_ld_wait_for(a1, c1);
+            if (j + 16 < kCorrTmemCols) {
+              tmem_ld_8cols(acc_tm + j + 16, a0);
+              tmem_ld_8cols(corr_tm + j + 16, c0);
+            } else {
+              release();
+            }
+            emit_t(j + 8, a1, c1);
+          }
+        }
+        if (row_ok && nt0 < p.N) {
+          const int ncols = p.N - nt0 < BN ? p.N - nt0 : BN;
+          fence_proxy_async_smem();  // the row's shared stores, visible to the bulk copy
+          bulk_store(static_cast<uint16_t*>(p.out) + static_cast<int64_t>(t) * p.ldo + nt0, orow_s,
+                     static_cast<uint32_t>(ncols) * 2, out_pol);
+          bulk_commit();
+        }
+      } else if (staged) {
+        // 32-bit outputs, rows that no bulk copy can write, and calls that want the accumulator: straight from
+        // registers.
+        const float sa = Sa[rl];
+        const float ob = kOneBlock ? Os[rl] : 0.f;
+        const uint32_t corr_tm = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kCorrCol0;
+        for (int c = 0; c < BN / CW; ++c) {
+          const int jc = c * CW;  // column within the tile
+          uint32_t acc[CW], cr[CW];
+          tmem_ld_16cols(acc_tm + jc, acc);
+          if (!kOneBlock && jc < kCorrTmemCols) tmem_ld_16cols(corr_tm + jc, cr);
+          tmem_ld_wait();
+          const int nb = nt0 + jc;
+          if (!row_ok || nb >= p.N) continue;
+          if (!kOneBlock && jc >= kCorrTmemCols) {
+#pragma unroll
+            for (int q4 = 0; q4 < CW / 4; ++q4) {
+              const uint4 v = lds128(orow_s + (jc - kCorrTmemCols) * 4 + 16 * q4);
               cr[4 * q4] = v.x; cr[4 * q4 + 1] = v.y; cr[4 * q4 + 2] = v.z; cr[4 * q4 + 3] = v.w;
             }
           }
@@ -533,9 +773,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
           float z[CW];
 #pragma unroll
           for (int jj = 0; jj < CW; ++jj) {
-            // (acc' - 8 Rt) 2^-18, then * 2^18: both steps exact.
-            const float accf = (__uint_as_float(acc[jj]) + Rt[jc + jj]) * kAccScale;
-            z[jj] = Ws[jc + jj] * fmaf(sa, accf, __uint_as_float(cr[jj]));
+            const float r8 = kOneBlock ? Rs[jc + jj] * -8.f : Rt[jc + jj];
+            const float corr = kOneBlock ? ob * Rs[jc + jj] : __uint_as_float(cr[jj]);
+            const float accf = fmaf(__uint_as_float(acc[jj]), kAccScale, r8);  // an exact integer
+            z[jj] = Ws[jc + jj] * fmaf(sa, accf, corr);
           }
           store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, z, nvalid, out_pol);
           if (p.acc_debug != nullptr) {
@@ -545,85 +786,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
               if (jj < nvalid) d[jj] = __float2int_rn(__uint_as_float(acc[jj]) * 262144.0f);
           }
         }
-      } else if (kOneBlock) {
-        // Packed fp32 pairs; each lane rounds as y = s_w * fma(s_a, acc * 2^18, o R)
-        // does, with acc = (acc' - 8 R) 2^-18 formed exactly first (s_a * 2^18 and
-        // its product with acc are exact). 16-bit rows go to shared memory and
-        // leave by one bulk copy per row once the accumulator is read, so the
-        // tile's output write overlaps the next tile's MMAs.
-        const float sa2 = Sa[rl] * kAccScale;
-        const float ob = Os[rl * kStageGp];
-        const uint64_t SA2 = pack2(sa2, sa2), OB = pack2(ob, ob);
-        const uint64_t M8 = pack2(-0x1p-15f, -0x1p-15f);  // -8 * 2^-18
-        const bool async_out = OUT != OFFQ_F32 && p.async_out != 0;
-        const uint32_t orow_s = base + SL::kOffOut + rl * kOutPitch;
-        if (async_out) bulk_wait_read_all();  // this row's previous copy has read the buffer
-        for (int c = 0; c < kEpiCols / CW; c += 2) {
-          uint32_t acc2[2 * CW];
-          tmem_ld_32cols_waited(acc_tm + c * CW, acc2);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t* acc = &acc2[h * CW];
-            const int nb = n0 + (c + h) * CW;
-            const int jc = half * kEpiCols + (c + h) * CW;
-            if (!row_ok || nb >= p.N) continue;
-            const int nvalid = p.N - nb < CW ? p.N - nb : CW;
-            const float4* r4 = reinterpret_cast<const float4*>(Rs + jc);
-            const float4* w4 = reinterpret_cast<const float4*>(Ws + jc);
-            float y[CW];
-#pragma unroll
-            for (int q4 = 0; q4 < CW / 4; ++q4) {
-              const float4 rv = r4[q4], wv = w4[q4];
-              const uint64_t R0 = pack2(rv.x, rv.y), R1 = pack2(rv.z, rv.w);
-              uint64_t A0 = pack2(__uint_as_float(acc[4 * q4]), __uint_as_float(acc[4 * q4 + 1]));
-              uint64_t A1 = pack2(__uint_as_float(acc[4 * q4 + 2]), __uint_as_float(acc[4 * q4 + 3]));
-              A0 = fma2v(R0, M8, A0);
-              A1 = fma2v(R1, M8, A1);
-              unpack2(mul2v(pack2(wv.x, wv.y), fma2v(SA2, A0, mul2v(OB, R0))), y[4 * q4], y[4 * q4 + 1]);
-              unpack2(mul2v(pack2(wv.z, wv.w), fma2v(SA2, A1, mul2v(OB, R1))), y[4 * q4 + 2], y[4 * q4 + 3]);
-            }
-            if (async_out) {
-              uint32_t hv[CW / 2];
-#pragma unroll
-              for (int i = 0; i < CW / 2; ++i) {
-                if (OUT == OFFQ_BF16) {
-                  const __nv_bfloat162 v = __floats2bfloat162_rn(y[2 * i], y[2 * i + 1]);
-                  hv[i] = *reinterpret_cast<const uint32_t*>(&v);
-                } else {
-                  const __half2 v = __floats2half2_rn(y[2 * i], y[2 * i + 1]);
-                  hv[i] = *reinterpret_cast<const uint32_t*>(&v);
-                }
-              }
-              sts128(orow_s + (c + h) * CW * 2, hv[0], hv[1], hv[2], hv[3]);
-              sts128(orow_s + (c + h) * CW * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
-            } else {
-              store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, y, nvalid, out_pol);
-            }
-            if (p.acc_debug != nullptr) {
-              int32_t* d = p.acc_debug + static_cast<int64_t>(t) * p.N + nb;
-#pragma unroll
-              for (int jj = 0; jj < CW; ++jj)
-                if (jj < nvalid) d[jj] = __float2int_rn(__uint_as_float(acc[jj]) * 262144.0f);
-            }
-          }
-        }
-        if (async_out && row_ok && n0 < p.N) {
-          const int ncols = p.N - n0 < kEpiCols ? p.N - n0 : kEpiCols;
-          fence_proxy_async_smem();  // the row's shared stores, visible to the bulk copy
-          bulk_store(static_cast<uint16_t*>(p.out) + static_cast<int64_t>(t) * p.ldo + n0, orow_s,
-                     static_cast<uint32_t>(ncols) * 2, out_pol);
-          bulk_commit();
-        }
       } else {
         // More offset blocks than the staging area holds: read the constants directly.
         const float sa = row_ok ? __ldg(p.a_scale + t) : 0.f;
         const bool has_off = p.a_offset != nullptr && row_ok;
         const float* orow = has_off ? p.a_offset + static_cast<int64_t>(t) * G : p.a_scale;
-        for (int c = 0; c < kEpiCols / CW; ++c) {
+        for (int c = 0; c < BN / CW; ++c) {
           uint32_t acc[CW];
           tmem_ld_16cols(acc_tm + c * CW, acc);
           tmem_ld_wait();
-          const int nb = n0 + c * CW;
+          const int nb = nt0 + c * CW;
           if (!row_ok || nb >= p.N) continue;
           const int nvalid = p.N - nb < CW ? p.N - nb : CW;
           float y[CW], a[CW];
@@ -657,13 +829,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
           }
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (ok && lane == 0) arrive_cluster(acc_empty_l);
+      if (ok && !released) release();
       epi_sync<kEpiWarps>();  // the staged constants are reused for the next tile
       if (*epi_stop) break;
     }
-    if (kOneBlock) bulk_wait_all();  // output rows in flight are written before the CTA ends
+    bulk_wait_all();  // output rows in flight are written before the CTA ends
   }
 
   // ---------------- teardown ----------------
@@ -755,7 +925,7 @@ GemmParams gemm_params(const uint8_t* a_codes, const float* a_scale, const float
   p.n_blocks = static_cast<int>((N + 31) / 32);
   p.kchunks = static_cast<int>(K / 32);
   p.vec_ok = aligned(w_offsum, 16) && aligned(w_scale, 16) && (N % 4 == 0);
-  p.async_out = out_dtype != OFFQ_F32 && N % 8 == 0;
+  p.async_out = out_dtype != OFFQ_F32 && N % 8 == 0 && acc_debug == nullptr;
   return p;
 }
 

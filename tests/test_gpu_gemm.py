@@ -368,3 +368,28 @@ def test_few_token_forms_agree():
             np.testing.assert_array_equal(acct, acc9[:t])
             np.testing.assert_array_equal(yt, y9[:t])
 
+
+@pytest.mark.parametrize("T,K,N,g,out_dt,ldo", [
+    (2943, 512, 1000, 512, "bf16", 1008),    # one offset block; a last pair tile with 127 rows, ragged columns
+    (3000, 512, 1000, 256, "f16", 1000),     # two blocks
+    (2817, 2752, 1008, 64, "bf16", 1016),    # 43 blocks, one row in the last tile
+    (2943, 1536, 1000, 32, "bf16", 1000),    # 48 blocks: the most that are staged
+    (2943, 1568, 1000, 32, "bf16", 1000),    # 49: read at the tile end
+    (3000, 2752, 1003, 64, "bf16", 1008),    # rows that no bulk copy can write
+    (2900, 2752, 1000, 64, "f32", 1000),
+])
+def test_pair_form_output_routes(T, K, N, g, out_dt, ldo):
+    """The 256 x 256 pair kernel's 16-bit rows leave through shared memory, or straight from registers when the
+    accumulator is asked for (which the oracle checks): the same bits, and nothing past the N columns."""
+    rows = np.r_[0:3, 127:130, 255:258, T - 2:T]
+    y_rows, _, _, w = _check_layer(T, K, N, g, out_dt, seed=T + K, ldo=ldo, rows=rows)
+    x = W.activations(T, K, seed=T + K, n_out=2, mult=50.0)
+    a_codes, a_scale, a_off = Q.quantize_act(torch.from_numpy(x).to(torch.bfloat16).cuda(), g)
+    w_codes, w_scale, rowsum = Q.prepare_weight(torch.from_numpy(w).cuda(), g)
+    args = (a_codes, a_scale, a_off, T, N, K, g, w_codes, w_scale, rowsum)
+    y = [torch.full((T, ldo), float("nan"), dtype=OUT_DT[out_dt], device="cuda") for _ in range(2)]
+    Q.offq_w4a4_linear(*args, y[0], ldo)
+    Q.offq_w4a4_linear(*args, y[1], ldo, torch.zeros((T, N), dtype=torch.int32, device="cuda"))
+    assert torch.equal(y[0][:, :N], y[1][:, :N])
+    assert bool(torch.isnan(y[0][:, N:]).all())
+    np.testing.assert_array_equal(y[0][rows, :N].double().cpu().numpy(), y_rows)
