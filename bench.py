@@ -751,7 +751,7 @@ def time_decode(device, args, flush_l2, stream):
     if st != Q.OFFQ_OK:
         raise RuntimeError(f"device status after the decode sweep: {Q.status_string(st)}")
     del sets
-    kern = "w4a4_few_kernel (T <= 32)" if best["T"] <= 32 else "w4a4_mid_kernel (tcgen05, 32 < T)"
+    kern = "w4a4_few_kernel (T <= 16)" if best["T"] <= 16 else "w4a4_mid_kernel (tcgen05, 16 < T)"
     out["roofline"] = {"bound": "hbm", "kernel": f"{kern} weight stream (T = {best['T']})",
                        "achieved": best["weight_gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
                        "frac": best["weight_frac"], "bytes": w_bytes}

@@ -158,7 +158,7 @@ int offq_quantize_act(const void* x, int x_dtype, int64_t T, int64_t K, int64_t 
  *           + s_w[n] * sum_b o[t][b] * R[b][n]
  *
  * accumulated exactly in integers (the tensor cores see both codes as exact
- * fp8 or, at T <= 32, fp16 values; every partial sum is an integer below 2^24
+ * fp8 or, in the few-token form, fp16 values; every partial sum is an integer below 2^24
  * times a power of two), dequantized in fp32
  * and rounded once to the output type.
  *
@@ -181,12 +181,12 @@ int offq_quantize_act(const void* x, int x_dtype, int64_t T, int64_t K, int64_t 
  *   acc_debug device, [T][N] int32 or NULL. When given, also receives the
  *             integer the tensor cores accumulate, sum_k (q_a + 8) * q_w
  *             (equal to the true dot product plus 8 * sum_k q_w[n][k]).
- * Forms: T <= 32 the few-token form (weights straight into registers,
- * warp-level MMA); above, the pair-tile tensor-core kernel, or, where its 256 x
- * 256 tiles are too few to fill the chip, the form that gives a CTA 128 output
- * channels x up to 128 tokens and splits K over a cluster. All give the same
- * accumulator and apply the same epilogue.
- * Ordering: the T <= 32 form starts reading w_codes, w_scale and w_offsum
+ * Forms: T <= 16, and smaller layers at T <= 32, the few-token form (weights
+ * straight into registers, warp-level MMA); else the pair-tile tensor-core
+ * kernel, or, where its 256 x 256 tiles are too few to fill the chip, the form
+ * that gives a CTA 128 output channels x up to 128 tokens and splits K over a
+ * cluster. All give the same accumulator and apply the same epilogue.
+ * Ordering: the few-token form starts reading w_codes, w_scale and w_offsum
  * before the kernel ahead of it in the stream has finished (programmatic
  * dependent launch), so they must not be written by a kernel that releases its
  * dependents early (ordinary kernels never do; no kernel of this library that

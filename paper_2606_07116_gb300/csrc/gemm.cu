@@ -949,11 +949,11 @@ extern "C" int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, co
     return OFFQ_ERR_MISALIGNED;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (T <= few_max_tokens())
-    return w4a4_linear_few(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype, ldo,
-                           acc_debug, s);
   if (mid_takes(T, N, K, K / g))
     return w4a4_linear_mid(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype, ldo,
+                           acc_debug, s);
+  if (T <= few_max_tokens())
+    return w4a4_linear_few(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype, ldo,
                            acc_debug, s);
   const GemmParams p = gemm_params(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype,
                                    ldo, acc_debug);

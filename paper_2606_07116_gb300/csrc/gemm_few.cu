@@ -5,8 +5,9 @@
 //   y[t][n] = s_w[n] * ( s_a[t] * (acc'[n][t] - 8 Rt[n]) + sum_b o[t][b] * R[b][n] ),
 //   acc'[n][t] = sum_k q_w[n][k] * (q_a[t][k] + 8),   Rt[n] = sum_b R[b][n].
 //
-// Few tokens (T <= 32): warp-level MMA (mma.sync m16n8k16, fp16 operands, fp32
-// accumulate).
+// Few tokens (T <= 32; from 17 on only layers small enough that the tcgen05
+// form of gemm_mid.cu is slower): warp-level MMA (mma.sync m16n8k16, fp16
+// operands, fp32 accumulate).
 //
 // The weights stream once from HBM and meet at most 32 tokens, so the time is
 // that stream plus the chain of latencies from the end of the kernel ahead

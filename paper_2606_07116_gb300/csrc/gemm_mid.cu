@@ -6,7 +6,8 @@
 //
 // Here the pair kernel's 256 x 256 tiles are too few to fill the chip (16 for
 // 4096 channels and up to 256 tokens, on 76 pairs), and each walks all of K.
-// So:
+// And from 17 tokens on, warp-level MMAs over all of a large layer's weights take
+// longer than this. So:
 //  * a CTA takes 128 output channels (the MMA's M side) x up to 128 tokens (N,
 //    a multiple of 16 near an equal share of the tokens) and, in a cluster of
 //    S = 1, 2, 4 or 8, an S-th of K; S is the largest that one wave holds. The
@@ -540,26 +541,36 @@ int launch_mid(const MidParams& p, int64_t ctas, size_t bytes, cudaStream_t s) {
 
 namespace offq {
 
-// Microseconds a call takes in this form and in the pair kernel's, fitted to both
-// forms measured over N = 512 .. 28672, K = 512 .. 28672 and 33 .. 1024 tokens
-// (weights past the L2): waves of CTAs (pairs), each of a fixed cost, a cost per
-// k-tile and one per offset block. The fit is within 20 % of either side there, and
-// where the two are closer than that it matters little which is taken: 512 x 4096
-// -> 4096 15.4 against 18.5; 201 x 4096 -> 11008 29.8 against 19.0.
+// Microseconds a call takes in this form and in its neighbours, fitted to all of
+// them measured over N = 512 .. 28672, K = 512 .. 28672 and 4 .. 1100 tokens
+// (weights past the L2). Here: waves of CTAs, each of a fixed cost, a cost per
+// k-tile and an exchange that grow with its tokens, and one per offset block.
+// The pair kernel: waves of 256 x 256 tiles, each bound by its MMAs or by its offset
+// correction. The few-token kernel with two token tiles: its warp-level MMAs over
+// all weights (with one tile, to 16 tokens, it is the faster one at most sizes and
+// at the others within 5 %). The fit is within 20 % of each side, and where two are
+// closer than that it matters little which is taken: 400 x 4096 -> 4096 15.2 here
+// against 17.4 in pairs; 201 x 4096 -> 11008 29.8 against 18.0; 257 x 11008 -> 4096
+// (43 blocks) 37.0 against 40.0, 1100 tokens 84.9 against 74.1; 32 x 8192 -> 16896
+// 19.5 against 30.2 few-token, 32 x 4096 -> 4096 8.2 against 6.0.
 bool mid_takes(int64_t T, int64_t N, int64_t K, int64_t G) {
+  constexpr int64_t kFewTile = 16;
   const int sms = mid_num_sms();
-  if (sms < 2) return false;
+  if (sms < 2 || T <= kFewTile) return false;
   const int64_t nk = (K + kMidBK - 1) / kMidBK;
   const int64_t tiles = (N + kMidM - 1) / kMidM * ((T + kMidMaxN - 1) / kMidMaxN);
   int64_t S = 1;
   while (S < 8 && split_fits(S * 2, tiles, nk, sms)) S *= 2;
+  const double k = static_cast<double>(nk), blocks = G > 1 ? static_cast<double>(G) : 0.0;
+  const double fill = static_cast<double>(T) / static_cast<double>((T + kMidMaxN - 1) / kMidMaxN * kMidMaxN);
+  const double exchange = S > 1 ? 5.6 + 2.0 * fill : 5.0;
   const double mid = static_cast<double>((tiles * S + sms - 1) / sms) *
-                     (0.33 * static_cast<double>(nk) / static_cast<double>(S) + (S > 1 ? 8.5 : 6.5) +
-                      (G > 1 ? 0.1 * static_cast<double>(G) : 0.0));
-  const int64_t pairs = (N + 255) / 256 * ((T + 255) / 256);
-  const double pair = static_cast<double>((pairs + sms / 2 - 1) / (sms / 2)) *
-                      (G > 1 ? 0.36 * static_cast<double>(nk) + 10.0 + 0.27 * static_cast<double>(G)
-                             : 0.28 * static_cast<double>(nk) + 9.0);
+                     ((0.21 + 0.12 * fill) * k / static_cast<double>(S) + exchange + 0.15 * blocks);
+  if (T <= few_max_tokens()) return mid < 2.0 + 2.5e-7 * static_cast<double>(N) * static_cast<double>(K);
+  const double waves = static_cast<double>(((N + 255) / 256 * ((T + 255) / 256) + sms / 2 - 1) / (sms / 2));
+  const double mma = 0.08 * k + waves * (0.31 * k + 2.0);
+  const double corr = G > 1 ? waves * (0.14 * k + 0.45 * blocks + 3.0) : 0.0;
+  const double pair = 3.0 + (mma > corr ? mma : corr);
   return mid < pair;
 }
 

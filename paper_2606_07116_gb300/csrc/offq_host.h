@@ -83,8 +83,8 @@ int few_max_tokens();
 int w4a4_linear_few(const uint8_t* a_codes, const float* a_scale, const float* a_offset, int64_t T, int64_t N,
                     int64_t K, int32_t g, const uint8_t* w_codes, const float* w_scale, const float* w_offsum,
                     void* out, int out_dtype, int64_t ldo, int32_t* acc_debug, cudaStream_t stream);
-// Form between decode and prefill (csrc/gemm_mid.cu): whether a shape takes it
-// (G offset blocks), and its launch.
+// Form between decode and prefill (csrc/gemm_mid.cu): whether a shape takes it,
+// before either other form (G offset blocks), and its launch.
 bool mid_takes(int64_t T, int64_t N, int64_t K, int64_t G);
 int w4a4_linear_mid(const uint8_t* a_codes, const float* a_scale, const float* a_offset, int64_t T, int64_t N,
                     int64_t K, int32_t g, const uint8_t* w_codes, const float* w_scale, const float* w_offsum,

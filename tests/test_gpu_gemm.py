@@ -159,6 +159,8 @@ def test_few_token_form(T, K, N, g, out_dt):
 
 
 @pytest.mark.parametrize("T,K,N,g,out_dt", [
+    (17, 4096, 12296, 4096, "bf16"), # the fewest tokens, no split of K
+    (31, 8192, 8200, 1024, "f32"),   # 17 to 32 tokens, K over two
     (33, 128, 40, 128, "f32"),       # one k-tile, 48 token columns, no split of K
     (40, 1056, 129, 32, "bf16"),     # a short last k-tile; one channel into a second tile; 33 offset blocks
     (65, 8192, 1000, 8192, "f16"),   # K over eight CTAs, 80 token columns (five chunks: three CTAs own none)
