@@ -211,6 +211,28 @@ __device__ __forceinline__ void tmem_st_16rows_32cols(uint32_t taddr, const uint
       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld_16rows_32cols(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Where column c of a tile lies so that a lane's 8 columns of 32 (2 m, 2 m + 1 of each 8) are 32 contiguous bytes.
+__device__ __forceinline__ int frag_pos(int c) { return (c & ~31) + (c & 6) * 4 + ((c >> 3) & 3) * 2 + (c & 1); }
+__device__ __forceinline__ void lds_4x64(const float* p, uint64_t (&v)[4]) {
+  const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(p), b = *reinterpret_cast<const ulonglong2*>(p + 4);
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+// Four 8 x 8 matrices of 16-bit values: lane l gives row l / 4, columns 2 (l % 4) and + 1 of matrix j in r[j], and in
+// addr the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&r)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3])
+               : "memory");
+}
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
@@ -475,8 +497,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
       if constexpr (kOneBlock) {
         for (int i = et; i < BN; i += kEpiWarps * 32) {
           const bool in = nt0 + i < p.N;
-          Rs[i] = in ? __ldg(p.rowsum + nt0 + i) : 0.f;
-          Ws[i] = in ? __ldg(p.w_scale + nt0 + i) : 0.f;
+          Rs[frag_pos(i)] = in ? __ldg(p.rowsum + nt0 + i) : 0.f;
+          Ws[frag_pos(i)] = in ? __ldg(p.w_scale + nt0 + i) : 0.f;
         }
         const bool in = m0 + et < p.T;
         Sa[et] = in ? __ldg(p.a_scale + m0 + et) : 0.f;
@@ -626,49 +648,62 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
         // before, of a tile's 30 k at K = 4096, now 2.9 k: 8192 tokens x 4096 -> 4096 98 -> 89 us, -> 11008 248 ->
         // 222 us; 14 blocks of 1024 -> 4096 at 2048 tokens (there with strided 32-byte stores) 93 -> 88 us.
         if constexpr (kOneBlock) {
+          // 16-lane x 256-bit fragments: a lane holds 4 rows x 8 columns of every 32, so R and s_w are read once per 4
+          // rows (one row per lane: 128 reads of 16 bytes each, now 32), and one stmatrix stores 8 rows x 32 columns.
+          // With one warp per sub-partition the drain's length is its instruction count: 2048 tokens x 4096 -> 4096
+          // 29.5 -> 28.9 us, x 8192 -> 28672 290.5 -> 285.0 (without stmatrix 29.2 and 287.7; scalar FMAs 30.5, 296.9).
           // Packed fp32 pairs; each lane rounds as y = s_w * fma(s_a, acc * 2^18, o R)
           // does, with acc = (acc' - 8 R) 2^-18 formed exactly first (s_a * 2^18 and
           // its product with acc are exact).
-          const float sa2 = Sa[rl] * kAccScale;
-          const float ob = Os[rl];
-          const uint64_t SA2 = pack2(sa2, sa2), OB = pack2(ob, ob);
+          const int q = lane >> 2, m = lane & 3;
           const uint64_t M8 = pack2(-0x1p-15f, -0x1p-15f);  // -8 * 2^-18
-          bulk_wait_read_all();  // this row's previous copy has read the buffer
-          auto emit = [&](int c, const uint32_t (&acc)[CW]) {
-            const float4* r4 = reinterpret_cast<const float4*>(Rs + c * CW);
-            const float4* w4 = reinterpret_cast<const float4*>(Ws + c * CW);
-            uint32_t hv[CW / 2];
+          float sa2[4], ob[4];  // rows q + 8 i
 #pragma unroll
-            for (int q4 = 0; q4 < CW / 4; ++q4) {
-              const float4 rv = r4[q4], wv = w4[q4];
-              const uint64_t R0 = pack2(rv.x, rv.y), R1 = pack2(rv.z, rv.w);
-              uint64_t A0 = pack2(__uint_as_float(acc[4 * q4]), __uint_as_float(acc[4 * q4 + 1]));
-              uint64_t A1 = pack2(__uint_as_float(acc[4 * q4 + 2]), __uint_as_float(acc[4 * q4 + 3]));
-              A0 = fma2v(R0, M8, A0);
-              A1 = fma2v(R1, M8, A1);
-              float y0, y1, y2, y3;
-              unpack2(mul2v(pack2(wv.x, wv.y), fma2v(SA2, A0, mul2v(OB, R0))), y0, y1);
-              unpack2(mul2v(pack2(wv.z, wv.w), fma2v(SA2, A1, mul2v(OB, R1))), y2, y3);
-              hv[2 * q4] = pack_out<OUT>(y0, y1);
-              hv[2 * q4 + 1] = pack_out<OUT>(y2, y3);
+          for (int i = 0; i < 4; ++i) {
+            sa2[i] = Sa[quarter * 32 + q + 8 * i] * kAccScale;
+            ob[i] = Os[quarter * 32 + q + 8 * i];
+          }
+          // This lane's row of the 8 x 8 matrices a stmatrix writes: row lane % 8, columns 8 (lane / 8).
+          const uint32_t frow_s = base + SL::kOffOut + (quarter * 32 + (lane & 7)) * kOutPitch + (lane >> 3) * 16;
+          bulk_wait_read_all();  // these rows' previous copies have read the buffer
+          __syncwarp();
+          uint64_t R[4], Wc[4];
+          // Rows q + 16 h, q + 16 h + 8 of 32 columns.
+          auto emit = [&](int sb, int h, const uint32_t (&acc)[CW]) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int r = 2 * h + i;
+              const uint64_t SA2 = pack2(sa2[r], sa2[r]), OB = pack2(ob[r], ob[r]);
+              uint32_t hv[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                uint64_t A = pack2(__uint_as_float(acc[4 * j + 2 * i]), __uint_as_float(acc[4 * j + 2 * i + 1]));
+                A = fma2v(R[j], M8, A);
+                float y0, y1;
+                unpack2(mul2v(Wc[j], fma2v(SA2, A, mul2v(OB, R[j]))), y0, y1);
+                hv[j] = pack_out<OUT>(y0, y1);
+              }
+              stmatrix4(frow_s + 8 * r * kOutPitch + sb * 64, hv);
             }
-            sts128(orow_s + c * CW * 2, hv[0], hv[1], hv[2], hv[3]);
-            sts128(orow_s + c * CW * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
           };
           uint32_t a0[CW], a1[CW];
-          tmem_ld_16cols(acc_tm, a0);
+          tmem_ld_16rows_32cols(acc_tm, a0);
 #pragma unroll
-          for (int c = 0; c < BN / CW; c += 2) {
+          for (int sb = 0; sb < BN / 32; ++sb) {
+            lds_4x64(Rs + sb * 32 + m * 8, R);
+            lds_4x64(Ws + sb * 32 + m * 8, Wc);
             tmem_ld_wait_for(a0);
-            tmem_ld_16cols(acc_tm + (c + 1) * CW, a1);
-            emit(c, a0);
+            tmem_ld_16rows_32cols(acc_tm + (16u << 16) + sb * 32, a1);
+            emit(sb, 0, a0);
             tmem_ld_wait_for(a1);
-            if (c + 2 < BN / CW)
-              tmem_ld_16cols(acc_tm + (c + 2) * CW, a0);
+            if (sb + 1 < BN / 32)
+              tmem_ld_16rows_32cols(acc_tm + (sb + 1) * 32, a0);
             else
               release();
-            emit(c + 1, a1);
+            emit(sb, 1, a1);
           }
+          fence_proxy_async_smem();  // a row's outputs come from four lanes and leave by one's bulk copy
+          __syncwarp();
         } else {
           // Several blocks: columns 128..255 first, from the highest down, because their outputs overwrite corrections
           // of higher columns of the row; then 0..127, whose corrections are in TMEM.
@@ -773,10 +808,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
           float z[CW];
 #pragma unroll
           for (int jj = 0; jj < CW; ++jj) {
-            const float r8 = kOneBlock ? Rs[jc + jj] * -8.f : Rt[jc + jj];
-            const float corr = kOneBlock ? ob * Rs[jc + jj] : __uint_as_float(cr[jj]);
+            const float r8 = kOneBlock ? Rs[frag_pos(jc + jj)] * -8.f : Rt[jc + jj];
+            const float corr = kOneBlock ? ob * Rs[frag_pos(jc + jj)] : __uint_as_float(cr[jj]);
             const float accf = fmaf(__uint_as_float(acc[jj]), kAccScale, r8);  // an exact integer
-            z[jj] = Ws[jc + jj] * fmaf(sa, accf, corr);
+            z[jj] = Ws[kOneBlock ? frag_pos(jc + jj) : jc + jj] * fmaf(sa, accf, corr);
           }
           store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, z, nvalid, out_pol);
           if (p.acc_debug != nullptr) {
