@@ -950,10 +950,10 @@ def run_gpu(args, rank, world, local_rank):
             "what": "the same layers in MXFP4 (E2M1 codes, a power-of-two scale per 32 channels) with the offsets "
                     "as zero-points: offq_quantize_act_mx + offq_mx_linear, no KV4",
             "value": round(job_tops(ops, world, m_ms), 3), "unit": UNIT, "ms_per_step": round(m_ms, 4),
-            "roofline": {"bound": "tensor", "kernel": "w4a4_gemm_kernel<MX> (tcgen05.mma kind::f8f6f4, codes "
-                                                      "widened with their block shifts in the converter warps)",
-                         "achieved": round(m_gemm_tflops, 2), "peak": round(fp8_peak, 1), "unit": "TFLOP/s",
-                         "frac": round(m_gemm_tflops / fp8_peak, 4), "gemm_ms_per_step": round(m_gemm_ms, 4)},
+            "roofline": {"bound": "tensor", "kernel": "mx_gemm_kernel (tcgen05.mma kind::mxf4, block-scaled FP4)",
+                         "achieved": round(m_gemm_tflops, 2), "peak": round(3.0 * fp8_peak, 1), "unit": "TFLOP/s",
+                         "peak_source": "the fp8 peak x the nominal fp4/fp8 ratio 3",
+                         "frac": round(m_gemm_tflops / (3.0 * fp8_peak), 4), "gemm_ms_per_step": round(m_gemm_ms, 4)},
             "act_quant": {"value": round(m_quant_gbs, 1), "unit": "GB/s", "peak": peaks["hbm_gbs"],
                           "frac": round(m_quant_gbs / peaks["hbm_gbs"], 4), "ms_per_step": round(m_quant_ms, 4),
                           "bytes_per_step": mstep.quant_bytes()},
