@@ -233,6 +233,11 @@ __device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&r)[4])
                "r"(r[2]), "r"(r[3])
                : "memory");
 }
+__device__ __forceinline__ uint64_t lds64(uint32_t addr) {
+  uint64_t v;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
@@ -266,12 +271,13 @@ __device__ __forceinline__ int b_block(const GemmParams& p, int tile, uint32_t r
 // Persistent pair kernel: cluster c processes pair tiles c, c + clusters, ...
 // (pair tile index mapped to (m-pair, n-tile) by tile_mn). The k-tile counter g runs
 // across tiles so the stage ring never drains between tiles.
-// kOneBlock: the offsets span the whole row (G == 1). kUnstaged: more than
-// kMaxStageG offset blocks, whose constants are read from global memory at the
-// tile end. Layers with several
-// offset blocks run a separate instantiation, so the register allocation of
-// the common one-block kernel does not carry the G-term epilogue loop.
-template <int OUT, bool kOneBlock, bool kUnstaged>
+// kOneBlock: the offsets span the whole row (G == 1). kWindows: more than
+// kMaxStageG offset blocks, staged in windows of that many (2048 tokens x 11904 ->
+// 4096 with 93 blocks 139 us; read from global memory at the tile end, 1537). Each
+// runs its own instantiation, so the register allocation of the common one-block
+// kernel does not carry the G-term epilogue loop, nor that of up to kMaxStageG
+// blocks the reload of a window's sums (6912 -> 2560, 27 blocks: 50 us, 56 with it).
+template <int OUT, bool kOneBlock, bool kWindows>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kThreads, 1)
     w4a4_gemm_kernel(const GemmParams p) {
   constexpr float kAccScale = 262144.0f;  // operands are integers times 2^-9: the accumulator carries 2^-18
@@ -473,9 +479,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
     const int quarter = warp & 3;              // TMEM lanes this warp may read
     const int et = threadIdx.x - kFirstEpi * 32;
     const int G = kOneBlock ? 1 : p.G;
-    // More offset blocks than the staging area holds take their own
-    // instantiation, so its register needs stay out of the staged kernels.
-    constexpr bool staged = !kUnstaged;
     float* Rs = reinterpret_cast<float*>(smem + kOffR);
     float* Ws = reinterpret_cast<float*>(smem + kOffW);
     float* Os = reinterpret_cast<float*>(smem + kOffO);
@@ -504,57 +507,59 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
         Sa[et] = in ? __ldg(p.a_scale + m0 + et) : 0.f;
         Os[et] = in && p.a_offset != nullptr ? __ldg(p.a_offset + m0 + et) : 0.f;
         epi_sync<kEpiWarps>();
-      } else if constexpr (staged) {
+      } else {
         // Asynchronous copies, so their latencies overlap: 9.5 k cycles at 43 blocks (22 k as loads into registers).
         // R: thread et takes columns 2 et and 2 et + 1 of every block, placed so that the 8 columns a lane multiplies
-        // below are 32 contiguous bytes.
+        // below are 32 contiguous bytes. More than kMaxStageG blocks come in windows, the correction carried on.
         const int c2 = 2 * et, n2 = nt0 + c2;
         float* rdst = Rs + (c2 & ~31) + (c2 & 7) * 4 + ((c2 >> 3) & 3) * 2;
+        Ws[c2] = n2 < p.N ? __ldg(p.w_scale + n2) : 0.f;
+        Ws[c2 + 1] = n2 + 1 < p.N ? __ldg(p.w_scale + n2 + 1) : 0.f;
+        Sa[et] = m0 + et < p.T ? __ldg(p.a_scale + m0 + et) : 0.f;
+        if (p.async_out) bulk_wait_read_all();  // this row's previous output copy has read the buffer
+        float rt0 = 0.f, rt1 = 0.f;
+        for (int b0 = 0; b0 < (kWindows ? G : 1); b0 += kMaxStageG) {
+        const int Gw = kWindows && G - b0 > kMaxStageG ? kMaxStageG : G - b0;  // blocks of this window
+        if (kWindows && b0 > 0) epi_sync<kEpiWarps>();  // the previous window has been read
         if (p.vec_ok && n2 < p.N) {
-          const float* src = p.rowsum + n2;
-          for (int b = 0; b < G; ++b, src += p.N) cp_async<8>(smem_u32(rdst + b * BN), src);
+          const float* src = p.rowsum + static_cast<int64_t>(b0) * p.N + n2;
+          for (int b = 0; b < Gw; ++b, src += p.N) cp_async<8>(smem_u32(rdst + b * BN), src);
         } else {
-          for (int b = 0; b < G; ++b) {
-            const float* src = p.rowsum + static_cast<int64_t>(b) * p.N + n2;
+          for (int b = 0; b < Gw; ++b) {
+            const float* src = p.rowsum + static_cast<int64_t>(b0 + b) * p.N + n2;
             rdst[b * BN] = n2 < p.N ? __ldg(src) : 0.f;
             rdst[b * BN + 1] = n2 + 1 < p.N ? __ldg(src + 1) : 0.f;
           }
         }
-        Ws[c2] = n2 < p.N ? __ldg(p.w_scale + n2) : 0.f;
-        Ws[c2 + 1] = n2 + 1 < p.N ? __ldg(p.w_scale + n2 + 1) : 0.f;
-        Sa[et] = m0 + et < p.T ? __ldg(p.a_scale + m0 + et) : 0.f;
         // Offsets, [b][row]: rows q, q + 8, q + 16, q + 24 of a 32-row group side by side.
-        const int64_t left = static_cast<int64_t>(p.T - m0) * G;  // offsets from row m0 on; not positive past the end
-        const float* o0 = p.a_offset + static_cast<int64_t>(m0) * G;
-        const int step_r = kEpiWarps * 32 / G, step_b = kEpiWarps * 32 - step_r * G;
-        int r = et / G, b = et - r * G;
-        for (int i = et; i < BM * G; i += kEpiWarps * 32) {
-          float* dst = Os + b * kOPitch + (r & ~31) + (r & 7) * 4 + ((r >> 3) & 3);
-          if (p.a_offset != nullptr && i < left)
-            cp_async<4>(smem_u32(dst), o0 + i);
-          else
-            *dst = 0.f;
-          r += step_r;
-          b += step_b;
-          if (b >= G) {
-            b -= G;
-            ++r;
+        {
+          const float* o0 = p.a_offset + static_cast<int64_t>(m0) * G + b0;
+          const int step_r = kEpiWarps * 32 / Gw, step_b = kEpiWarps * 32 - step_r * Gw;
+          int r = et / Gw, b = et - r * Gw;
+          while (r < BM) {
+            float* dst = Os + b * kOPitch + (r & ~31) + (r & 7) * 4 + ((r >> 3) & 3);
+            if (p.a_offset != nullptr && m0 + r < p.T)
+              cp_async<4>(smem_u32(dst), o0 + static_cast<int64_t>(r) * G + b);
+            else
+              *dst = 0.f;
+            r += step_r;
+            b += step_b;
+            if (b >= Gw) {
+              b -= Gw;
+              ++r;
+            }
           }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
-        {
-          // Rt[n] = -8 sum_b R[b][n]: integers, exact in fp32. (This thread's own copies.)
-          float r0 = 0.f, r1 = 0.f;
+        // Rt[n] = -8 sum_b R[b][n]: integers, exact in fp32. (This thread's own copies.)
 #pragma unroll 4
-          for (int bb = 0; bb < G; ++bb) {
-            const float2 v = *reinterpret_cast<const float2*>(rdst + bb * BN);
-            r0 += v.x;
-            r1 += v.y;
-          }
-          Rt[c2] = r0 * -8.f;
-          Rt[c2 + 1] = r1 * -8.f;
+        for (int bb = 0; bb < Gw; ++bb) {
+          const float2 v = *reinterpret_cast<const float2*>(rdst + bb * BN);
+          rt0 += v.x;
+          rt1 += v.y;
         }
-        if (p.async_out) bulk_wait_read_all();  // this row's previous output copy has read the buffer
+        Rt[c2] = rt0 * -8.f;
+        Rt[c2 + 1] = rt1 * -8.f;
         epi_sync<kEpiWarps>();
         // While this tile's MMAs run: its offset correction, per element the same chain as at the tile end (block 0
         // multiplied, then FMAs in block order). A lane takes 4 rows x 8 columns at a time, the fragment that a
@@ -569,7 +574,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
         for (int sb = 0; sb < BN / 32; ++sb) {
           const float* rp = Rs + sb * 32 + m * 8;
           uint64_t y[4][4];  // [row q + 8 i][column pair 8 j + 2 m]
-          {
+          const uint32_t tm = corr_tm + sb * 32;
+          const uint32_t sm = corr_s + (sb * 32 - kCorrTmemCols) * 4;
+          int bb = 0;
+          if (!kWindows || b0 == 0) {
             const float4 o = *reinterpret_cast<const float4*>(op);
             const float4 ra = *reinterpret_cast<const float4*>(rp), rb = *reinterpret_cast<const float4*>(rp + 4);
             const uint64_t R[4] = {pack2(ra.x, ra.y), pack2(ra.z, ra.w), pack2(rb.x, rb.y), pack2(rb.z, rb.w)};
@@ -578,9 +586,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
             for (int i = 0; i < 4; ++i)
 #pragma unroll
               for (int j = 0; j < 4; ++j) y[i][j] = mul2v(O[i], R[j]);
+            bb = 1;
+          } else if (sb * 32 < kCorrTmemCols) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t u[16];
+              tmem_ld_16rows_32cols(tm + (static_cast<uint32_t>(16 * h) << 16), u);
+              tmem_ld_wait_for(u);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                y[2 * h][j] = pack2(__uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]));
+                y[2 * h + 1][j] = pack2(__uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]));
+              }
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) y[i][j] = lds64(sm + 8 * i * kOutPitch + 32 * j);
           }
 #pragma unroll 2
-          for (int bb = 1; bb < G; ++bb) {
+          for (; bb < Gw; ++bb) {
             const float4 o = *reinterpret_cast<const float4*>(op + bb * kOPitch);
             const float4 ra = *reinterpret_cast<const float4*>(rp + bb * BN);
             const float4 rb = *reinterpret_cast<const float4*>(rp + bb * BN + 4);
@@ -603,7 +629,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
                 u[4 * j] = __float_as_uint(v0); u[4 * j + 1] = __float_as_uint(v1);
                 u[4 * j + 2] = __float_as_uint(v2); u[4 * j + 3] = __float_as_uint(v3);
               }
-              tmem_st_16rows_32cols(corr_tm + (static_cast<uint32_t>(16 * h) << 16) + sb * 32, u);
+              tmem_st_16rows_32cols(tm + (static_cast<uint32_t>(16 * h) << 16), u);
             }
           } else {
 #pragma unroll
@@ -612,12 +638,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
               for (int j = 0; j < 4; ++j) {
                 float v0, v1;
                 unpack2(y[i][j], v0, v1);
-                sts64(corr_s + 8 * i * kOutPitch + (sb * 32 - kCorrTmemCols + 8 * j) * 4, __float_as_uint(v0),
-                      __float_as_uint(v1));
+                sts64(sm + 8 * i * kOutPitch + 32 * j, __float_as_uint(v0), __float_as_uint(v1));
               }
           }
         }
         tmem_st_wait();
+        }
         __syncwarp();  // a row's correction comes from four lanes
       }
       const bool ok = __all_sync(0xFFFFFFFFu, wait_cluster(acc_full, lt & 1, abort));
@@ -637,7 +663,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
         released = true;
       };
       const uint32_t orow_s = base + SL::kOffOut + rl * kOutPitch;
-      const bool async_out = OUT != OFFQ_F32 && !kUnstaged && p.async_out != 0;
+      const bool async_out = OUT != OFFQ_F32 && p.async_out != 0;
       if (!ok) {
         // Aborted: nothing to drain.
       } else if (async_out) {
@@ -783,7 +809,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
                      static_cast<uint32_t>(ncols) * 2, out_pol);
           bulk_commit();
         }
-      } else if (staged) {
+      } else {
         // 32-bit outputs, rows that no bulk copy can write, and calls that want the accumulator: straight from
         // registers.
         const float sa = Sa[rl];
@@ -814,48 +840,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
             z[jj] = Ws[kOneBlock ? frag_pos(jc + jj) : jc + jj] * fmaf(sa, accf, corr);
           }
           store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, z, nvalid, out_pol);
-          if (p.acc_debug != nullptr) {
-            int32_t* d = p.acc_debug + static_cast<int64_t>(t) * p.N + nb;
-#pragma unroll
-            for (int jj = 0; jj < CW; ++jj)
-              if (jj < nvalid) d[jj] = __float2int_rn(__uint_as_float(acc[jj]) * 262144.0f);
-          }
-        }
-      } else {
-        // More offset blocks than the staging area holds: read the constants directly.
-        const float sa = row_ok ? __ldg(p.a_scale + t) : 0.f;
-        const bool has_off = p.a_offset != nullptr && row_ok;
-        const float* orow = has_off ? p.a_offset + static_cast<int64_t>(t) * G : p.a_scale;
-        for (int c = 0; c < BN / CW; ++c) {
-          uint32_t acc[CW];
-          tmem_ld_16cols(acc_tm + c * CW, acc);
-          tmem_ld_wait();
-          const int nb = nt0 + c * CW;
-          if (!row_ok || nb >= p.N) continue;
-          const int nvalid = p.N - nb < CW ? p.N - nb : CW;
-          float y[CW], a[CW];
-#pragma unroll
-          for (int jj = 0; jj < CW; ++jj) {
-            y[jj] = 0.f;
-            a[jj] = __uint_as_float(acc[jj]);
-          }
-          for (int b = 0; b < G; ++b) {
-            const float ob = has_off ? __ldg(orow + b) : 0.f;
-            const float* rb = p.rowsum + static_cast<int64_t>(b) * p.N + nb;
-#pragma unroll
-            for (int jj = 0; jj < CW; ++jj)
-              if (jj < nvalid) {
-                const float r = __ldg(rb + jj);
-                y[jj] = fmaf(ob, r, y[jj]);
-                a[jj] = fmaf(r, -0x1p-15f, a[jj]);  // acc' - 8 R, in units of 2^-18: exact
-              }
-          }
-#pragma unroll
-          for (int jj = 0; jj < CW; ++jj) {
-            const float accf = a[jj] * kAccScale;
-            y[jj] = jj < nvalid ? __ldg(p.w_scale + nb + jj) * fmaf(sa, accf, y[jj]) : 0.f;
-          }
-          store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, y, nvalid, out_pol);
           if (p.acc_debug != nullptr) {
             int32_t* d = p.acc_debug + static_cast<int64_t>(t) * p.N + nb;
 #pragma unroll
@@ -898,12 +882,12 @@ int num_sms() {
   return sms[dev];
 }
 
-template <int OUT, bool kOneBlock, bool kUnstaged>
+template <int OUT, bool kOneBlock, bool kWindows>
 int launch_gemm(const GemmParams& p, cudaStream_t s) {
-  auto kern = w4a4_gemm_kernel<OUT, kOneBlock, kUnstaged>;
+  auto kern = w4a4_gemm_kernel<OUT, kOneBlock, kWindows>;
   constexpr int kThreads = Roles<kOneBlock>::kThreads;
   constexpr int kSmemBytes = Smem<kOneBlock>::kBytes;
-  if (!smem_optin<w4a4_gemm_kernel<OUT, kOneBlock, kUnstaged>>(kSmemBytes)) return OFFQ_ERR_CUDA;
+  if (!smem_optin<w4a4_gemm_kernel<OUT, kOneBlock, kWindows>>(kSmemBytes)) return OFFQ_ERR_CUDA;
   const int sms = num_sms();
   if (sms < 2) return OFFQ_ERR_CUDA;
   const int tiles = p.m_pairs * p.n_tiles;
@@ -912,20 +896,20 @@ int launch_gemm(const GemmParams& p, cudaStream_t s) {
 }
 
 int dispatch_gemm(const GemmParams& p, int out_dtype, cudaStream_t s) {
-  const bool unstaged = p.G > kMaxStageG;
+  const bool windows = p.G > kMaxStageG;
   switch (out_dtype) {
     case OFFQ_F32:
       return p.G == 1 ? launch_gemm<OFFQ_F32, true, false>(p, s)
-                      : unstaged ? launch_gemm<OFFQ_F32, false, true>(p, s)
-                                 : launch_gemm<OFFQ_F32, false, false>(p, s);
+             : windows ? launch_gemm<OFFQ_F32, false, true>(p, s)
+                       : launch_gemm<OFFQ_F32, false, false>(p, s);
     case OFFQ_BF16:
       return p.G == 1 ? launch_gemm<OFFQ_BF16, true, false>(p, s)
-                      : unstaged ? launch_gemm<OFFQ_BF16, false, true>(p, s)
-                                 : launch_gemm<OFFQ_BF16, false, false>(p, s);
+             : windows ? launch_gemm<OFFQ_BF16, false, true>(p, s)
+                       : launch_gemm<OFFQ_BF16, false, false>(p, s);
     case OFFQ_F16:
       return p.G == 1 ? launch_gemm<OFFQ_F16, true, false>(p, s)
-                      : unstaged ? launch_gemm<OFFQ_F16, false, true>(p, s)
-                                 : launch_gemm<OFFQ_F16, false, false>(p, s);
+             : windows ? launch_gemm<OFFQ_F16, false, true>(p, s)
+                       : launch_gemm<OFFQ_F16, false, false>(p, s);
     default: return OFFQ_ERR_INVALID_ARG;
   }
 }

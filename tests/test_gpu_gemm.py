@@ -376,7 +376,8 @@ def test_few_token_forms_agree():
     (3000, 512, 1000, 256, "f16", 1000),     # two blocks
     (2817, 2752, 1008, 64, "bf16", 1016),    # 43 blocks, one row in the last tile
     (2943, 1536, 1000, 32, "bf16", 1000),    # 48 blocks: the most that are staged
-    (2943, 1568, 1000, 32, "bf16", 1000),    # 49: read at the tile end
+    (2943, 1568, 1000, 32, "bf16", 1000),    # 49: a second window of one block
+    (2900, 3104, 1000, 32, "f16", 1000),     # 97: three windows
     (3000, 2752, 1003, 64, "bf16", 1008),    # rows that no bulk copy can write
     (2900, 2752, 1000, 64, "f32", 1000),
 ])
