@@ -108,6 +108,7 @@ struct MxGemmParams {
   int m_pairs, n_tiles, raster_m;
   int t_blocks, n_blocks;  // 32-row blocks present in the code buffers
   int staged;              // row sums and offsets go through shared memory
+  int vec_r;               // rows of the row sums allow 16-byte reads
   int async_out;           // 16-bit output and N % 8 == 0: rows leave by bulk copy
 };
 
@@ -457,6 +458,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
                 y2[2 * q + 1] = fma2v(O2, pack2(rv.z, rv.w), y2[2 * q + 1]);
               }
             }
+          } else if (p.vec_r && nb + CW <= p.N && p.a_offset != nullptr) {
+            // Too many blocks to stage: R by 16-byte reads, several blocks' in flight (one element at a time was the
+            // larger part of such a layer: 2 x 18944 -> 7808 with 148 blocks 875 us, now 357).
+            const float* o = p.a_offset + static_cast<int64_t>(row_ok ? t : 0) * G;
+            const float4* r4 = reinterpret_cast<const float4*>(p.rowsum + nb);
+            const int64_t pitch = p.N / 4;
+            {
+              const float ob = __ldg(o);
+              const uint64_t O2 = pack2(ob, ob);
+#pragma unroll
+              for (int q = 0; q < CW / 4; ++q) {
+                const float4 rv = __ldg(r4 + q);
+                y2[2 * q] = mul2v(O2, pack2(rv.x, rv.y));
+                y2[2 * q + 1] = mul2v(O2, pack2(rv.z, rv.w));
+              }
+            }
+#pragma unroll 4
+            for (int b = 1; b < G; ++b) {
+              const float ob = __ldg(o + b);
+              const uint64_t O2 = pack2(ob, ob);
+#pragma unroll
+              for (int q = 0; q < CW / 4; ++q) {
+                const float4 rv = __ldg(r4 + b * pitch + q);
+                y2[2 * q] = fma2v(O2, pack2(rv.x, rv.y), y2[2 * q]);
+                y2[2 * q + 1] = fma2v(O2, pack2(rv.z, rv.w), y2[2 * q + 1]);
+              }
+            }
           } else {
             float z[CW];
 #pragma unroll
@@ -620,6 +648,7 @@ extern "C" int offq_mx_linear(const uint8_t* a_codes, const uint8_t* a_shifts, c
   p.t_blocks = static_cast<int>((T + 31) / 32);
   p.n_blocks = static_cast<int>((N + 31) / 32);
   p.staged = p.G <= kXMaxG;
+  p.vec_r = aligned(w_offsum, 16) && N % 4 == 0;
   p.async_out = out_dtype != OFFQ_F32 && N % 8 == 0;
   CUtensorMap amap, wmap;
   if (!encode_codes(&amap, a_codes, p.t_blocks, K / 32, kXABlocks) ||
