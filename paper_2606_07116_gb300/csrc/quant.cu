@@ -776,6 +776,13 @@ __global__ void __launch_bounds__(WideGeo<L>::kMaxThreads) quantize_rows_wide_ke
 // absmax crosses warps through shared memory (one barrier per row group).
 constexpr int k1kMaxWarps = 28;
 
+// Buffers of the warps' row maxima, taken in turn by row group. A warp writes its
+// maximum, passes the group's one barrier and reads all the row's. With one buffer
+// nothing would stand between a slow warp's read and a fast warp's write for the
+// next group; with two, that write goes elsewhere, and the one after it comes behind
+// the next group's barrier, which the slow warp reaches only after its read.
+constexpr int kRowMaxBufs = 2;
+
 template <typename Tin>
 __device__ __forceinline__ float smem_elem(const Tin* p) {
   if constexpr (sizeof(Tin) == 4) {
@@ -837,7 +844,7 @@ template <typename Tin>
 __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(const QuantArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int abort_flag;
-  __shared__ float wmax[k1kMaxWarps];
+  __shared__ float wmax[kRowMaxBufs][k1kMaxWarps];
   const int K = a.K, G = a.G, R = a.rows_per_cta;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lrow = warp / G;
@@ -854,6 +861,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
   // Rows fit an int here (the launcher checks), so group and row indices are 32-bit.
   const int ngroups = static_cast<int>((a.rows + R - 1) / R);
   int grp = blockIdx.x;
+  int turn = 0;  // of the row maxima's buffers
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int k = 0; k < ring.S; ++k) mbar_init(ring.bar0 + 8u * k, 1);
@@ -927,7 +935,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
       mx1 = fmax3(mx1, fabsf(v[i + 1].x), fabsf(v[i + 1].y));
     }
     const uint32_t wm = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(mx0, mx1)));
-    if (lane == 0) wmax[warp] = __uint_as_float(wm);
+    if (lane == 0) wmax[turn][warp] = __uint_as_float(wm);
     // One barrier per row group: the warps' maxima are visible, every thread has read
     // the slot (so it takes the group S turns ahead), and a wait that ran out anywhere
     // in the CTA is seen by all.
@@ -939,7 +947,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
     if (threadIdx.x == 0 && next < ngroups) ring_issue<Tin>(a, next, R, ring.slot(), ring.bar());
     ring.advance();
     const float m = __uint_as_float(
-        __reduce_max_sync(0xFFFFFFFFu, lane < G ? __float_as_uint(wmax[lrow * G + lane]) : 0u));
+        __reduce_max_sync(0xFFFFFFFFu, lane < G ? __float_as_uint(wmax[turn][lrow * G + lane]) : 0u));
     const float inv = m > 0.f ? __fdiv_rn(7.0f, m) : 0.f;
 
     const float2 inv2 = make_float2(inv, inv), mag2 = make_float2(kMagic8, kMagic8);
@@ -960,6 +968,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
       if (b == 0 && lane == 0) a.scale[row] = m * a.scale_mul;
       if (lane == 0 && a.offset != nullptr) a.offset[static_cast<int64_t>(row) * G + b] = offs ? off * a.inv_sqrt_g : 0.f;
     }
+    turn = turn + 1 == kRowMaxBufs ? 0 : turn + 1;
     grp += gridDim.x;
     if (grp >= ngroups) break;
   }
