@@ -296,6 +296,10 @@ struct RowRing {
   uint32_t phase;
   __device__ __forceinline__ uint8_t* slot() const { return base + static_cast<size_t>(s) * slot_bytes; }
   __device__ __forceinline__ uint32_t bar() const { return bar0 + 8u * static_cast<uint32_t>(s); }
+  // The parity of the group's index i: s is i mod S and phase (i / S) mod 2.
+  __device__ __forceinline__ uint32_t turn() const {
+    return (static_cast<uint32_t>(s) + (static_cast<uint32_t>(S) & phase)) & 1u;
+  }
   __device__ __forceinline__ void advance() {
     if (++s == S) {
       s = 0;
@@ -861,7 +865,6 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
   // Rows fit an int here (the launcher checks), so group and row indices are 32-bit.
   const int ngroups = static_cast<int>((a.rows + R - 1) / R);
   int grp = blockIdx.x;
-  int turn = 0;  // of the row maxima's buffers
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int k = 0; k < ring.S; ++k) mbar_init(ring.bar0 + 8u * k, 1);
@@ -935,6 +938,7 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
       mx1 = fmax3(mx1, fabsf(v[i + 1].x), fabsf(v[i + 1].y));
     }
     const uint32_t wm = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(mx0, mx1)));
+    const uint32_t turn = ring.turn();
     if (lane == 0) wmax[turn][warp] = __uint_as_float(wm);
     // One barrier per row group: the warps' maxima are visible, every thread has read
     // the slot (so it takes the group S turns ahead), and a wait that ran out anywhere
@@ -968,7 +972,6 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
       if (b == 0 && lane == 0) a.scale[row] = m * a.scale_mul;
       if (lane == 0 && a.offset != nullptr) a.offset[static_cast<int64_t>(row) * G + b] = offs ? off * a.inv_sqrt_g : 0.f;
     }
-    turn = turn + 1 == kRowMaxBufs ? 0 : turn + 1;
     grp += gridDim.x;
     if (grp >= ngroups) break;
   }
@@ -1026,8 +1029,8 @@ template <typename Tin, bool kRot, bool kGen>
 __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(const QuantArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int abort_flag;
-  __shared__ float wpart[k1kMaxWarps];  // per-warp block sums (no rotation, g > 1024)
-  __shared__ int wmaxx[k1kMaxWarps];    // per-warp largest block exponent (+ 1024)
+  __shared__ float wpart[k1kMaxWarps];             // per-warp block sums (no rotation, g > 1024)
+  __shared__ int wmaxx[kRowMaxBufs][k1kMaxWarps];  // per-warp largest block exponent (+ 1024)
   const int K = a.K, R = a.rows_per_cta;
   const int nbw = kGen ? (K + 1023) / 1024 : K / 1024;  // warps per row
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1205,7 +1208,8 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
     constexpr int kUnnorm = kRot && !kGen ? 5 : 0;  // values are 2^5 r with the rotation over g = 1024
     const int xl = amax > 0.f ? floor_log2(amax) - 2 - kUnnorm : -1000;
     const uint32_t wx = __reduce_max_sync(0xFFFFFFFFu, static_cast<uint32_t>(xl + 1024));
-    if (lane == 0) wmaxx[warp] = static_cast<int>(wx);
+    const uint32_t turn = ring.turn();
+    if (lane == 0) wmaxx[turn][warp] = static_cast<int>(wx);
     if (!__syncthreads_and(ok)) {
       ring_fail(ring, grp, ngroups, a.status);
       return;
@@ -1213,7 +1217,8 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_mx_1k_kernel(con
     const int next = grp + ring.S * static_cast<int>(gridDim.x);
     if (threadIdx.x == 0 && next < ngroups) ring_issue<Tin>(a, next, R, ring.slot(), ring.bar());
     ring.advance();
-    int xmax = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, lane < nbw ? static_cast<uint32_t>(wmaxx[lrow * nbw + lane]) : 0u)) - 1024;
+    const uint32_t wrow = lane < nbw ? static_cast<uint32_t>(wmaxx[turn][lrow * nbw + lane]) : 0u;
+    int xmax = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, wrow)) - 1024;
     if (xmax < -900) xmax = 0;  // an all-zero row: any exponent
     const int xlo = xmax - 6;
     const int X = xl > xlo ? xl : xlo;

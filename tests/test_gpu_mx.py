@@ -240,3 +240,28 @@ def test_mx_quantizer_spans(T, K, g, rotate, dt):
     code, sh, X = _decode(codes, shifts, scale, T, K)
     check_mx(code, X, ref, xe, g, rotate)
     assert not off.any()
+
+
+@pytest.mark.parametrize("T,K,g,rotate,dt", [
+    (2048, 11008, 256, True, "bf16"),    # 11 warps a row, the last span ragged; rotations within a span
+    (2048, 11008, 256, False, "bf16"),   # block means over 8 lanes
+    (5001, 1152, 128, True, "f16"),      # two rows of two warps per CTA, a ragged last group
+    (5001, 1152, 128, False, "f32"),
+    (1500, 8192, 8192, True, "bf16"),    # rotation over eight warps
+    (2000, 6144, 2048, True, "f32"),     # over two warps of six
+])
+def test_mx_quantizer_general_form_over_many_rows(T, K, g, rotate, dt):
+    """The general span form with several row groups per CTA: ring slots, their phases and the buffers of
+    the row maxima are used again. Neighbouring rows differ by powers of four, so a row coded with another
+    row's exponent is far off."""
+    x = W.activations(T, K, seed=T + K + g, n_out=3, mult=60.0)
+    x *= (4.0 ** (np.arange(T) % 5 - 2)).astype(np.float32)[:, None]
+    xe, codes, shifts, scale, off = _quant(x, g, rotate, dt)
+    rows = np.unique(np.concatenate([W.unit_index_sample(T, 160, seed=17), [0, 1, T - 2, T - 1]]))
+    ref = O.quantize_act_mx(xe[rows], g, rotate=rotate, offset=True)
+    code, sh, X = _decode(codes, shifts, scale, T, K)
+    check_mx(code[rows], X[rows], ref, xe[rows], g, rotate)
+    check_offsets(off.cpu().numpy()[rows], ref["offset"], xe[rows], g, rotate)
+    # Every row: its largest block exponent is the one its scale was made from.
+    assert np.all((sh >= 0) & (sh <= O.MX_SPAN))
+    assert np.all(sh.max(axis=1) == O.MX_SPAN)

@@ -62,12 +62,24 @@ def test_one_buffer_is_overtaken():
     assert violations(3, 2, 1)
 
 
-@pytest.mark.parametrize("kernel,array", [("quantize_rows_1k_kernel", "wmax")])
+@pytest.mark.parametrize("kernel,array", [("quantize_rows_1k_kernel", "wmax"),
+                                          ("quantize_mx_1k_kernel", "wmaxx")])
 def test_kernels_take_enough_buffers_in_turn(kernel, array):
     body, bufs = _kernel_source(kernel)
     assert not violations(2, 4, bufs)
     assert not violations(3, 3, bufs)
-    # The array has that many buffers, every access names the group's, and the turn moves on once per group.
+    # The array has that many buffers, and every access names the group's.
     uses = re.findall(rf"\b{array}(\[[^\]]*\])", body)
-    assert uses[0] == "[kRowMaxBufs]" and len(uses) >= 3 and all(u == "[turn]" for u in uses[1:])
-    assert body.count("turn = turn + 1 == kRowMaxBufs ? 0 : turn + 1;") == 1
+    assert uses[0] == "[kRowMaxBufs]" and len(uses) == 3 and all(u == "[turn]" for u in uses[1:])
+    assert bufs == 2 and body.count("const uint32_t turn = ring.turn();") == 1
+
+
+@pytest.mark.parametrize("S", [1, 2, 3])
+def test_ring_turn_is_the_parity_of_the_group(S):
+    """RowRing::turn() from the slot and its phase."""
+    s = phase = 0
+    for i in range(6 * S):
+        assert (s + (S & phase)) & 1 == i & 1
+        s += 1
+        if s == S:
+            s, phase = 0, phase ^ 1
