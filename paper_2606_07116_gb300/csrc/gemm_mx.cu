@@ -187,7 +187,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
   auto empty = [&](int s) { return bar0 + 8u * (2 * kXStages + s); };  // both: stage s consumed
   auto acc_full = [&](int b) { return bar0 + 8u * (3 * kXStages + b); };       // both: accumulator b complete
   auto acc_empty = [&](int b) { return bar0 + 8u * (3 * kXStages + 2 + b); };  // leader: accumulator b drained
-  const uint32_t done = bar0 + 8u * (3 * kXStages + 4);                // both, after an abort: MMAs finished
+  const uint32_t done = bar0 + 8u * (3 * kXStages + 4);                // leader, after an abort: MMAs finished
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kXOffMisc);
   volatile int* abort = reinterpret_cast<volatile int*>(smem + kXOffMisc + 16);
   volatile int* epi_stop = reinterpret_cast<volatile int*>(smem + kXOffMisc + 32);
@@ -281,9 +281,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
           }
         }
       }
-      // After an abort, the teardown's sign that the MMAs already issued are done.
-      if (elect_one()) mma2_commit_both(done);
-      __syncwarp();
     }
   } else if (warp >= kXFirstSf && warp < kXFirstEpi) {
     // ---------------- scales: shift words -> UE8M0 in tensor memory ----------------
@@ -558,7 +555,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
       for (int u = loads > kXStages ? loads - kXStages : 0; u < loads; ++u)
         wait_teardown(full(u % kXStages), (u / kXStages) & 1);
     }
-    if (warp == 1 && rank == 0) wait_teardown(done, 0);
+    if (warp == 1 && rank == 0) {
+      // The MMAs this warp issued are done when a commit after them arrives. Only here, and only at this CTA's barrier:
+      // without an abort every accumulator has been waited for, and an arrival that nobody waits for could reach a CTA
+      // that has ended.
+      if (elect_one()) mma2_commit(done);
+      __syncwarp();
+      wait_teardown(done, 0);
+    }
   }
   tc_fence_before();
   __syncthreads();

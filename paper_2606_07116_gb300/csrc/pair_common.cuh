@@ -120,6 +120,11 @@ __device__ __forceinline__ void mma2_commit_both(uint32_t bar) {
       : "memory");
 }
 
+// As mma2_commit_both, but arrives on this CTA's barrier only.
+__device__ __forceinline__ void mma2_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void tmem_st_32cols(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "

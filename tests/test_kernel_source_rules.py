@@ -1,0 +1,35 @@
+"""Rules of the CUDA sources that no run can show to be kept: what they guard against depends on how
+the compiler places an instruction, or on two SMs' timing."""
+
+import os
+import re
+
+from paper_2606_07116_gb300 import build as B
+
+
+def source(name):
+    """A source file without its comments."""
+    with open(os.path.join(B.CSRC, name)) as f:
+        text = f.read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def block(text, start):
+    """The braced block that begins at or after `start`."""
+    a = text.index("{", start)
+    depth = 0
+    for i in range(a, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[a:i + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def test_mx_gemm_commits_its_teardown_barrier_only_after_an_abort():
+    """An arrival that nobody waits for may reach a CTA that has ended: the commit to `done` belongs to the
+    abort's teardown, goes to the issuer's own CTA, and is waited for there."""
+    text = source("gemm_mx.cu")
+    commits = re.findall(r"mma2_commit\w*\(done\)", text)
+    assert commits == ["mma2_commit(done)"]
+    teardown = block(text, text.index("if (*abort) {"))
+    assert teardown.index("mma2_commit(done)") < teardown.index("wait_teardown(done, 0)")
