@@ -178,22 +178,6 @@ __device__ __forceinline__ void tile_mn(const GemmParams& p, int tile, int& mp, 
   mp = grp * p.raster_m + (local - nt * gm);
 }
 
-// Waits for the TMEM loads into r; the statement also hands the registers on, so
-// nothing reads them before it.
-__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&a)[8], uint32_t (&b)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
-               :
-               : "memory");
-}
 __device__ __forceinline__ void tmem_ld_8cols(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -820,7 +804,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
           uint32_t acc[CW], cr[CW];
           tmem_ld_16cols(acc_tm + jc, acc);
           if (!kOneBlock && jc < kCorrTmemCols) tmem_ld_16cols(corr_tm + jc, cr);
-          tmem_ld_wait();
+          tmem_ld_wait_for(acc);
+          if (!kOneBlock && jc < kCorrTmemCols) tmem_ld_wait_for(cr);
           const int nb = nt0 + jc;
           if (!row_ok || nb >= p.N) continue;
           if (!kOneBlock && jc >= kCorrTmemCols) {

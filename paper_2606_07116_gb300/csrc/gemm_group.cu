@@ -447,7 +447,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
               for (int c = 0; c < kGScCols / 16; ++c) {
                 uint32_t pv[16];
                 tmem_ld_16cols(lane_base + b * GBN + c * 16, pv);
-                tmem_ld_wait();
+                tmem_ld_wait_for(pv);
                 if (c == kGScCols / 16 - 1) {
                   // The partial is in registers: its buffer may take another group.
                   tc_fence_before();

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
         if (d == rank) continue;
         uint32_t v[kMidChunk];
         tmem_ld_16cols(lane_tm + c * kMidChunk, v);
-        tmem_ld_wait();
+        tmem_ld_wait_for(v);
         const int src = rank < d ? rank : rank - 1;
         const uint32_t dst = cluster_addr(base + p.off_red, d) +
                              (src * max_own + c - d * nch / S) * kMidChunkBytes;

@@ -498,7 +498,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
 #pragma unroll
             for (int i = 0; i < CW / 2; ++i) y2[i] = pack2(z[2 * i], z[2 * i + 1]);
           }
-          tmem_ld_wait();
+          tmem_ld_wait_for(acc);
           if (!row_ok || nb >= p.N) continue;
           const uint64_t SA2 = pack2(sa, sa);
           float y[CW];

@@ -339,35 +339,22 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
-// Waits for this thread's TMEM loads; the registers they fill are operands, so
-// no use of them moves above the wait.
-__device__ __forceinline__ void tmem_wait_into(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :
-               : "memory");
-}
-
 // The four 32-column chunks of this thread's 128-column TMEM row: f(v, c) on
 // chunk c while chunk c + 1 is loading; last() once all four are loaded.
 template <typename F, typename G>
 __device__ __forceinline__ void tmem_row_pass(uint32_t row_tm, F&& f, G&& last) {
   uint32_t va[32], vb[32];
   tmem_ld_32cols(row_tm, va);
-  tmem_wait_into(va);
+  tmem_ld_wait_for(va);
   tmem_ld_32cols(row_tm + 32, vb);
   f(va, 0);
-  tmem_wait_into(vb);
+  tmem_ld_wait_for(vb);
   tmem_ld_32cols(row_tm + 64, va);
   f(vb, 1);
-  tmem_wait_into(va);
+  tmem_ld_wait_for(va);
   tmem_ld_32cols(row_tm + 96, vb);
   f(va, 2);
-  tmem_wait_into(vb);
+  tmem_ld_wait_for(vb);
   last();
   f(vb, 3);
 }
@@ -615,7 +602,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
       if constexpr (REFLECT) {
         uint32_t dv[16];
         tmem_ld_16cols(row_tm + kHd, dv);
-        tmem_ld_wait();
+        tmem_ld_wait_for(dv);
         const float d = (__uint_as_float(dv[0]) + __uint_as_float(dv[1])) + __uint_as_float(dv[2]);  // x . w
         nd2 = pack2(-2.f * d, -2.f * d);
       }

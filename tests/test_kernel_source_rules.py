@@ -33,3 +33,14 @@ def test_mx_gemm_commits_its_teardown_barrier_only_after_an_abort():
     assert commits == ["mma2_commit(done)"]
     teardown = block(text, text.index("if (*abort) {"))
     assert teardown.index("mma2_commit(done)") < teardown.index("wait_teardown(done, 0)")
+
+
+def test_waits_for_tensor_memory_loads_name_their_registers():
+    """A tcgen05.wait::ld that does not list the loaded registers orders memory accesses only: the compiler may
+    move or spill them before their data is there. Each wait is in the load's own statement or takes them as
+    operands."""
+    for name in sorted(os.listdir(B.CSRC)):
+        text = source(name)
+        for m in re.finditer(r"tcgen05\.wait::ld", text):
+            statement = text[text.rindex("asm volatile(", 0, m.start()):text.index(";\n}", m.end())]
+            assert "tcgen05.ld." in statement or '"+r"(' in statement, (name, statement)
