@@ -807,7 +807,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
           tmem_ld_wait_for(acc);
           if (!kOneBlock && jc < kCorrTmemCols) tmem_ld_wait_for(cr);
           const int nb = nt0 + jc;
-          if (!row_ok || nb >= p.N) continue;
+          if (nb >= p.N) break;
           if (!kOneBlock && jc >= kCorrTmemCols) {
 #pragma unroll
             for (int q4 = 0; q4 < CW / 4; ++q4) {
@@ -824,13 +824,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
             const float accf = fmaf(__uint_as_float(acc[jj]), kAccScale, r8);  // an exact integer
             z[jj] = Ws[kOneBlock ? frag_pos(jc + jj) : jc + jj] * fmaf(sa, accf, corr);
           }
-          store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, z, nvalid, out_pol);
-          if (p.acc_debug != nullptr) {
+          if (row_ok) store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, z, nvalid, out_pol);
+          if (row_ok && p.acc_debug != nullptr) {
             int32_t* d = p.acc_debug + static_cast<int64_t>(t) * p.N + nb;
 #pragma unroll
             for (int jj = 0; jj < CW; ++jj)
               if (jj < nvalid) d[jj] = __float2int_rn(__uint_as_float(acc[jj]) * 262144.0f);
           }
+          __syncwarp();  // the next columns' load needs every lane
         }
       }
       if (ok && !released) release();

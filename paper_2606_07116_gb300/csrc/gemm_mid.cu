@@ -350,16 +350,17 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
       for (int c = part; c < nch; c += kMidParts) {
         int d = 0;
         while ((d + 1) * nch / S <= c) ++d;  // the owner of chunk c
-        if (d == rank) continue;
-        uint32_t v[kMidChunk];
-        tmem_ld_16cols(lane_tm + c * kMidChunk, v);
-        tmem_ld_wait_for(v);
-        const int src = rank < d ? rank : rank - 1;
-        const uint32_t dst = cluster_addr(base + p.off_red, d) +
-                             (src * max_own + c - d * nch / S) * kMidChunkBytes;
+        if (d != rank) {
+          uint32_t v[kMidChunk];
+          tmem_ld_16cols(lane_tm + c * kMidChunk, v);
+          tmem_ld_wait_for(v);
+          const int src = rank < d ? rank : rank - 1;
+          const uint32_t dst = cluster_addr(base + p.off_red, d) +
+                               (src * max_own + c - d * nch / S) * kMidChunkBytes;
 #pragma unroll
-        for (int i = 0; i < kMidChunk / 4; ++i)
-          st_cluster_v4(dst + red_off(row, i), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+          for (int i = 0; i < kMidChunk / 4; ++i)
+            st_cluster_v4(dst + red_off(row, i), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
       }
     }
     cluster_arrive();
@@ -387,6 +388,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
     for (int h = part; h < (ch1 - ch0) * 2; h += kMidParts) {
       const int col = ch0 * kMidChunk + h * 8;  // within the tile
       const int tok0 = t0 + col;
+      __syncwarp();  // the load needs every lane; channels past the end took other branches
       uint32_t av[8];
       tmem_ld_8cols(lane_tm + col, av);
       float acc[8], cv[8];

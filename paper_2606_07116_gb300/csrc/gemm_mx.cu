@@ -486,9 +486,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
             float z[CW];
 #pragma unroll
             for (int i = 0; i < CW; ++i) z[i] = 0.f;
-            if (row_ok && p.a_offset != nullptr) {
+            if (p.a_offset != nullptr) {
               for (int b = 0; b < G; ++b) {
-                const float ob = __ldg(p.a_offset + static_cast<int64_t>(t) * G + b);
+                const float ob = __ldg(p.a_offset + static_cast<int64_t>(row_ok ? t : 0) * G + b);
                 const float* rb = p.rowsum + static_cast<int64_t>(b) * p.N + nb;
 #pragma unroll
                 for (int i = 0; i < CW; ++i)
@@ -499,7 +499,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
             for (int i = 0; i < CW / 2; ++i) y2[i] = pack2(z[2 * i], z[2 * i + 1]);
           }
           tmem_ld_wait_for(acc);
-          if (!row_ok || nb >= p.N) continue;
           const uint64_t SA2 = pack2(sa, sa);
           float y[CW];
           const float4* w4 = reinterpret_cast<const float4*>(Ws + jc);
@@ -511,7 +510,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
             unpack2(mul2v(pack2(wv.x, wv.y), fma2v(SA2, A0, y2[2 * q])), y[4 * q], y[4 * q + 1]);
             unpack2(mul2v(pack2(wv.z, wv.w), fma2v(SA2, A1, y2[2 * q + 1])), y[4 * q + 2], y[4 * q + 3]);
           }
-          if (async_out) {
+          if (async_out) {  // rows past the tokens too: they are not copied out
             uint32_t hv[CW / 2];
 #pragma unroll
             for (int i = 0; i < CW / 2; ++i) {
@@ -525,10 +524,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
             }
             sts128(orow_s + c * 2, hv[0], hv[1], hv[2], hv[3]);
             sts128(orow_s + c * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
-          } else {
+          } else if (row_ok) {
             const int nvalid = p.N - nb < CW ? p.N - nb : CW;
             store_out<OUT, CW>(p.out, static_cast<int64_t>(t) * p.ldo + nb, y, nvalid, out_pol);
           }
+          __syncwarp();  // the next columns' load needs every lane
         }
         tc_fence_before();
         __syncwarp();

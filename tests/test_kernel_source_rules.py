@@ -44,3 +44,22 @@ def test_waits_for_tensor_memory_loads_name_their_registers():
         for m in re.finditer(r"tcgen05\.wait::ld", text):
             statement = text[text.rindex("asm volatile(", 0, m.start()):text.index(";\n}", m.end())]
             assert "tcgen05.ld." in statement or '"+r"(' in statement, (name, statement)
+
+
+def test_loops_over_tensor_memory_columns_keep_the_warp_together():
+    """The .sync.aligned TMEM loads need all lanes of the warp at once. In a loop that issues them, lanes without a
+    row or a channel to write take no `continue`, and the warp meets again before the next load."""
+    for name in sorted(os.listdir(B.CSRC)):
+        text = source(name)
+        loops = [(m.start(), block(text, text.index(")", m.end()))) for m in re.finditer(r"\bfor \(", text)
+                 if re.match(r"for \([^{};]*;[^{};]*;[^{}]*?\) \{", text[m.start():])]
+        for start, body in loops:
+            inner = [b for _, b in loops if b in body and b != body]
+            own = body
+            for b in inner:
+                own = own.replace(b, "")
+            if not re.search(r"\btmem_ld_\w+\(", own):
+                continue
+            assert "continue;" not in own, (name, own[:200])
+            if "store_out<" in own or "p.out)" in own:
+                assert re.search(r"__syncwarp\(\)|__all_sync\(", own), (name, own[:200])
