@@ -186,11 +186,12 @@ int offq_quantize_act(const void* x, int x_dtype, int64_t T, int64_t K, int64_t 
  * kernel, or, where its 256 x 256 tiles are too few to fill the chip, the form
  * that gives a CTA 128 output channels x up to 128 tokens and splits K over a
  * cluster. All give the same accumulator and apply the same epilogue.
- * Ordering: the few-token form starts reading w_codes, w_scale and w_offsum
- * before the kernel ahead of it in the stream has finished (programmatic
- * dependent launch), so they must not be written by a kernel that releases its
- * dependents early (ordinary kernels never do; no kernel of this library that
- * finishes weights does).
+ * Ordering: at T <= 4 (with T' * K <= 98304, T' = T rounded up to 1, 2 or 4) the
+ * few-token form starts reading w_codes, w_scale and w_offsum before the kernel
+ * ahead of it in the stream has finished (programmatic dependent launch), so
+ * they must not be written by a kernel that releases its dependents early
+ * (ordinary kernels never do; nor does any kernel of this library that finishes
+ * a table of the weights). With more tokens nothing is read that early.
  */
 int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, const float* a_offset,
                      int64_t T, int64_t N, int64_t K, int32_t g,

@@ -26,20 +26,22 @@
 //    need the operands in shared or tensor memory first: a pipeline whose fill
 //    alone took longer than this whole kernel (14.3 us for 4096 x 4096 at 8
 //    tokens, against 3.6 here);
-//  * 8 warps split K. Each keeps two k-steps (4 KB) of weight codes in flight;
-//    the first two, the block row sums and an L2 prefetch of the CTA's
-//    remaining codes are issued before the wait for the kernel ahead
-//    (programmatic dependent launch), which makes the activations, not the
-//    weights: no kernel of this library that writes weight codes releases its
-//    dependents early;
+//  * 8 warps split K. Each keeps two k-steps (4 KB) of weight codes in flight.
+//    Prefetches of the CTA's weights into L2 are issued before the wait for the
+//    kernel ahead (programmatic dependent launch), and up to 4 tokens the first
+//    two k-steps' loads and the constants' as well: that kernel makes the
+//    activations, not the weights, and the caller keeps to it (offq.h). From 5
+//    tokens on nothing but the prefetch of the codes comes before the wait (4096
+//    -> 4096 at 5 tokens 4.0 us, with early loads 3.7; prefetching the scales and
+//    row sums too was slower at most sizes);
 //  * the token codes come through a small cp.async ring per warp (no barrier);
 //  * the warps' partial sums (exact in any order) meet in shared memory, and
 //    each warp finishes whole tokens, lane = output channel.
 // Measured per call, back to back over weight copies past the L2 (before: dp4a
-// up to 4 tokens, tcgen05 above): 4096 -> 4096 3.6 / 3.6 / 4.5 / 6.0 us at 1 /
-// 8 / 16 / 32 tokens (7.1 / 14.3 / 14.4 / 15.0); 4096 -> 11008 7.2 / 7.4 / 9.8 /
-// 13.7 (7.9 / 14.8 / 15.0 / 15.5); 11008 -> 4096 with 43 offset blocks 8.7 / 9.1 /
-// 10.3 / 14.5 (22.3 / 38.0 / 38.6 / 53.9). What bounds it: 1.6 us of launch and
+// up to 4 tokens, tcgen05 above): 4096 -> 4096 3.6 / 4.0 / 4.5 / 6.1 us at 1 /
+// 8 / 16 / 32 tokens (7.1 / 14.3 / 14.4 / 15.0); 4096 -> 11008 6.8 / 7.3 / 10.5 at
+// 1 / 8 / 16 (7.9 / 14.8 / 15.0); 11008 -> 4096 with 43 offset blocks 8.2 / 8.8 /
+// 10.3 / 14.2 (22.3 / 38.0 / 38.6 / 53.9). What bounds it: 1.6 us of launch and
 // dependency per call, then the latency of two weight loads per warp; above 8
 // tokens the mask-and-shift work per token.
 #include <cuda.h>
@@ -119,7 +121,7 @@ __device__ __forceinline__ void few_cp_async4(uint32_t dst, const void* src) {
 __device__ __forceinline__ void few_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // NT: 8-token tiles per CTA (and warp); kFewWarps warps split K. CTAS: CTAs per
-// SM the registers are budgeted for.
+// SM the registers are budgeted for. EARLY (of the kernel): reads_early().
 template <int NT, int CTAS>
 struct Few {
   static constexpr int KS = kFewWarps;
@@ -133,7 +135,7 @@ struct Few {
   static constexpr int kMain = KS * kRing > kRedFloats * 4 ? KS * kRing : kRedFloats * 4;
 };
 
-template <int OUT, int NT, int CTAS>
+template <int OUT, int NT, int CTAS, bool EARLY>
 __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const FewParams p) {
   using F = Few<NT, CTAS>;
   constexpr int KS = F::KS;
@@ -161,29 +163,45 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
   };
   uint32_t off = static_cast<uint32_t>(s0) * 2048u + static_cast<uint32_t>(t * 512 + g * 16);
   uint4 wv[F::kPdW][4];
+  auto first_w = [&] {
 #pragma unroll
-  for (int i = 0; i < F::kPdW; ++i) load_w(off + i * 2048u, wv[i]);
-  if (threadIdx.x == 0) {
-    const int bytes = kc * 512 < kFewL2Bytes ? kc * 512 : kFewL2Bytes;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(wblk), "r"(bytes) : "memory");
-  }
-  const float sw = n < p.N ? __ldg(p.w_scale + n) : 0.f;
-  if (p.staged) {
-    for (int i = threadIdx.x; i < p.G * 32; i += KS * 32) {
-      const int nn = rb * 32 + (i & 31);
-      if (nn < p.N)
-        few_cp_async4(smem_u32(sR + i), p.rowsum + static_cast<int64_t>(i >> 5) * p.N + nn);
-      else
-        sR[i] = 0.f;
+    for (int i = 0; i < F::kPdW; ++i) load_w(off + i * 2048u, wv[i]);
+  };
+  // Each warp asks the L2 for its own share of K, so all warps' first steps come first (one request
+  // for the CTA's whole block delivers the last warp's first codes after everyone else's last ones:
+  // 4096 -> 4096 at 17 tokens 6.7 us against 6.0, 11008 -> 4096 at 1 token 8.7 against 8.2).
+  auto prefetch_w = [&] {
+    const int c0 = 4 * s0, c1 = 4 * s1 < kc ? 4 * s1 : kc;
+    if (lane == 0 && c0 < c1) {
+      const int bytes = (c1 - c0) * 512 < kFewL2Bytes / KS ? (c1 - c0) * 512 : kFewL2Bytes / KS;
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(wblk + c0 * 512), "r"(bytes) : "memory");
     }
-  }
-  griddep_wait();
-  griddep_launch_dependents();
-
-  if (p.staged && p.a_offset != nullptr) {
-    const int cnt = p.T * p.G;
-    for (int i = threadIdx.x; i < cnt; i += KS * 32)
-      few_cp_async4(smem_u32(sO + i), p.a_offset + i);
+  };
+  // The epilogue's constants: the channel's scale, and the block row sums.
+  float sw;
+  auto constants = [&] {
+    sw = n < p.N ? __ldg(p.w_scale + n) : 0.f;
+    if (p.staged) {
+      for (int i = threadIdx.x; i < p.G * 32; i += KS * 32) {
+        const int nn = rb * 32 + (i & 31);
+        if (nn < p.N)
+          few_cp_async4(smem_u32(sR + i), p.rowsum + static_cast<int64_t>(i >> 5) * p.N + nn);
+        else
+          sR[i] = 0.f;
+      }
+    }
+  };
+  if constexpr (EARLY) {
+    first_w();
+    prefetch_w();
+    constants();
+    griddep_wait();
+    griddep_launch_dependents();
+  } else {
+    prefetch_w();
+    griddep_wait();
+    first_w();
+    griddep_launch_dependents();
   }
   // The warp's token codes: a ring of k-steps, chunk c of step s as kTokens rows
   // of 16 bytes. Lane l copies 16-byte pieces l, l + 32, ... of a step's 4 chunks.
@@ -204,6 +222,12 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
   };
 #pragma unroll
   for (int i = 0; i < F::kPdA - 1; ++i) copy_a(s0 + i, i);
+  if constexpr (!EARLY) constants();  // they join the next group of copies
+  if (p.staged && p.a_offset != nullptr) {
+    const int cnt = p.T * p.G;
+    for (int i = threadIdx.x; i < cnt; i += KS * 32)
+      few_cp_async4(smem_u32(sO + i), p.a_offset + i);
+  }
   // Scales of the tokens this warp finishes: lane i holds token ks + KS i.
   const int my_tok = ks + KS * lane;
   const float sa_l = ks + KS * lane < F::kTokens && my_tok < p.T ? __ldg(p.a_scale + my_tok) : 0.f;
@@ -329,21 +353,31 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
 // stream, and three CTAs (80 registers) keep it fuller (4096 -> 11008: 7.3 us against 8.1 with
 // two); up to two blocks per SM, two CTAs (128 registers) have the shorter chain (8192 x 28672:
 // 24.5 us against 37.0; 4096 x 4096: 3.6 against 3.8).
-template <int OUT, int NT, int CTAS>
+template <int OUT, int NT, int CTAS, bool EARLY>
 int launch_few(FewParams p, cudaStream_t s) {
   using F = Few<NT, CTAS>;
   p.staged = p.G <= kFewStageG && F::kTokens * p.G <= kFewStageO;
   const size_t bytes = F::kMain + (p.staged ? p.G * 32 + F::kTokens * p.G : 0) * sizeof(float);
-  if (!smem_optin<w4a4_few_kernel<OUT, NT, CTAS>>(F::kMain + (kFewStageG * 32 + kFewStageO) * 4)) return OFFQ_ERR_CUDA;
+  if (!smem_optin<w4a4_few_kernel<OUT, NT, CTAS, EARLY>>(F::kMain + (kFewStageG * 32 + kFewStageO) * 4)) return OFFQ_ERR_CUDA;
   const dim3 grid((p.N + 31) / 32);
-  return launch_pdl(w4a4_few_kernel<OUT, NT, CTAS>, grid, dim3(kFewWarps * 32), bytes, s, p);
+  return launch_pdl(w4a4_few_kernel<OUT, NT, CTAS, EARLY>, grid, dim3(kFewWarps * 32), bytes, s, p);
 }
 
 template <int OUT>
-int dispatch_few(const FewParams& p, bool many_blocks, cudaStream_t s) {
-  if (p.T <= 8) return many_blocks ? launch_few<OUT, 1, 3>(p, s) : launch_few<OUT, 1, 2>(p, s);
-  if (p.T <= 16) return launch_few<OUT, 2, 2>(p, s);
-  return launch_few<OUT, 4, 2>(p, s);
+int dispatch_few(const FewParams& p, bool many_blocks, bool early, cudaStream_t s) {
+  if (early) return many_blocks ? launch_few<OUT, 1, 3, true>(p, s) : launch_few<OUT, 1, 2, true>(p, s);
+  if (p.T <= 8) return many_blocks ? launch_few<OUT, 1, 3, false>(p, s) : launch_few<OUT, 1, 2, false>(p, s);
+  if (p.T <= 16) return launch_few<OUT, 2, 2, false>(p, s);
+  return launch_few<OUT, 4, 2, false>(p, s);
+}
+
+// Whether the weights may be read before the kernel ahead has finished, which asks of the caller
+// that it does not write them and release its dependents early: the calls that offq.h lists, and
+// no others.
+constexpr int kEarlyTokens = 4;
+constexpr int64_t kEarlyActs = 96 * 1024;
+bool reads_early(int64_t T, int64_t K) {
+  return T <= kEarlyTokens && (T > 2 ? kEarlyTokens : T) * K <= kEarlyActs;
 }
 
 int few_num_sms() {
@@ -384,11 +418,12 @@ int w4a4_linear_few(const uint8_t* a_codes, const float* a_scale, const float* a
   p.N = static_cast<int>(N);
   p.G = static_cast<int>(K / g);
   p.kchunks = static_cast<int>(K / 32);
+  const bool early = reads_early(T, K);
   const bool many = (N + 31) / 32 > 2 * sms;
   switch (out_dtype) {
-    case OFFQ_F32: return dispatch_few<OFFQ_F32>(p, many, stream);
-    case OFFQ_BF16: return dispatch_few<OFFQ_BF16>(p, many, stream);
-    case OFFQ_F16: return dispatch_few<OFFQ_F16>(p, many, stream);
+    case OFFQ_F32: return dispatch_few<OFFQ_F32>(p, many, early, stream);
+    case OFFQ_BF16: return dispatch_few<OFFQ_BF16>(p, many, early, stream);
+    case OFFQ_F16: return dispatch_few<OFFQ_F16>(p, many, early, stream);
     default: return OFFQ_ERR_INVALID_ARG;
   }
 }

@@ -25,8 +25,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch. Kernels are launched so that the next kernel
 // in the stream may be scheduled before this one ends; each kernel waits for
-// the grids it depends on before its first global-memory access, so only
-// launch latency and setup overlap.
+// the grids it depends on before it reads what they may write or writes
+// anything, so launch latency and setup overlap (and L2 prefetches of weights,
+// and the first reads of the weights in the few-token GEMM at up to 4 tokens).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

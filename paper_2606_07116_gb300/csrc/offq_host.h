@@ -36,8 +36,11 @@ inline int launch_status() {
 
 // Launches kern<<<grid, block, smem, stream>>>(args...) with programmatic
 // stream serialization: the kernel may be scheduled while the previous kernel
-// in the stream finishes, and waits for it (griddepcontrol.wait) before its
-// first global-memory access. Returns the launch's status.
+// in the stream finishes, and waits for it (griddepcontrol.wait) before it
+// reads what that kernel may write or writes anything. Prefetches into L2 may
+// come before the wait, and so do the weights' first reads in the few-token
+// GEMM at up to 4 tokens.
+// Returns the launch's status.
 template <typename... KArgs, typename... Args>
 inline int launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                       Args&&... args) {

@@ -2004,8 +2004,8 @@ __device__ __forceinline__ uint32_t weight_word(uint32_t u) {
 // 4096 x 14336 fp32, g = 1024, rotated: 67.9 us with it; a thread per (row,
 // block) walking 4-byte words 512 bytes apart made that 371.7 us,
 // sector-bound.)
-// It does not release its dependents early: the few-token GEMM starts reading
-// weight codes and row sums before it waits for the kernel ahead of it.
+// It does not release its dependents early: up to 4 tokens the GEMM starts
+// reading the weights before it waits for the kernel ahead of it.
 constexpr int kRepackWarps = 8;
 __global__ void __launch_bounds__(kRepackWarps * 32) weight_repack_kernel(uint8_t* __restrict__ codes,
                                                                           float* __restrict__ rowsum, int64_t N,

@@ -63,3 +63,27 @@ def test_loops_over_tensor_memory_columns_keep_the_warp_together():
             assert "continue;" not in own, (name, own[:200])
             if "store_out<" in own or "p.out)" in own:
                 assert re.search(r"__syncwarp\(\)|__all_sync\(", own), (name, own[:200])
+
+
+def test_few_token_gemm_reads_early_only_what_its_contract_names():
+    """Before the wait for the kernel ahead the few-token GEMM may read the weights (codes, scales, row sums) only
+    in the EARLY instantiation (offq.h names those calls), else only prefetch them, and touches nothing else of
+    its inputs."""
+    text = source("gemm_few.cu")
+    body = block(text, text.index("w4a4_few_kernel(const FewParams p)"))
+    for f, reads in (("first_w", "load_w("), ("constants", "p.w_scale")):
+        own = block(body, body.index(f"auto {f} = [&]"))
+        assert reads in own
+        body = body.replace(own, "")
+    load = body[body.index("auto load_w = "):]
+    body = body.replace(block(load, 0), "")
+    start = body.index("if constexpr (EARLY) {")
+    early = block(body, start)
+    late = block(body, start + len("if constexpr (EARLY) ") + len(early))
+    assert early.index("first_w();") < early.index("griddep_wait();") > early.index("constants();")
+    before, after = late.split("griddep_wait();")
+    assert "first_w();" in after and not re.search(r"first_w\(\)|constants\(\)|__ldg|cp_async|p\.a_|p\.out", before)
+    assert before.count(";") == 1 and "prefetch_w();" in before
+    head = body[:start]
+    assert not re.search(r"first_w\(\)|constants\(\)|__ldg|few_cp_async|p\.(a_\w+|out|w_scale|rowsum)\b", head)
+    assert re.search(r"return T <= kEarlyTokens && ", text)
