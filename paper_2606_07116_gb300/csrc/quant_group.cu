@@ -198,10 +198,12 @@ __global__ void __launch_bounds__(kMaxQWarps * 32) quantize_group_kernel(const G
 // interleaved sign-magnitude layout: per 8 channels in bytes B0..B3, Bj holds
 // |q(c_2j)| in bits 0-2 with its sign in bit 7, |q(c_2j+1)| in bits 4-6, and
 // in bit 3 the sign of q(c_(2j-1) mod 8).
+// Offline, and it finishes a table of the weights, so it does not release its
+// dependents early: for group == g the sums are offq_w4a4_linear's w_offsum,
+// which that call may read before it waits for the kernel ahead of it.
 __global__ void weight_group_sums_kernel(const uint8_t* __restrict__ codes, float* __restrict__ sums, int64_t N,
                                          int K, int group) {
   griddep_wait();
-  griddep_launch_dependents();
   const int Gq = K / group;
   const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (id >= N * Gq) return;

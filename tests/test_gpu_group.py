@@ -220,3 +220,27 @@ def test_group_gemm_zero_points_outside_the_code_range():
 def test_group_gemm_windows(T, K, N, out_dt):
     """The group GEMM at the edges of its windows of s, z and R, its tiles and their copies' alignment."""
     _check_group_layer(T, K, N, 128, out_dt, False, seed=T + K, ldo=(N + 7) // 8 * 8)
+
+
+@pytest.mark.parametrize("T", [1, 4, 5, 32])
+def test_group_sums_feed_the_linear_behind_them(T):
+    """For group == g the weight group sums are the per-token linear's row sums. The linear follows them on the
+    stream at once, through one buffer whose table changes with the weights: it must see the finished table."""
+    N, K, g = 8192, 4096, 128
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    ac, asc, aoff = Q.quantize_act(torch.randn((T, K), generator=gen, device="cuda").to(torch.bfloat16), g)
+    weights = [Q.prepare_weight(torch.randn((N, K), generator=gen, device="cuda") * 0.02, g) for _ in range(4)]
+    table = torch.zeros((K // g, N), device="cuda")
+    got = [torch.empty((T, N), device="cuda") for _ in range(12)]
+    want = [torch.empty((T, N), device="cuda") for _ in weights]
+    for i, out in enumerate(got):
+        wc, wsc, _ = weights[i % 4]
+        Q.offq_weight_group_sums(wc, N, K, g, table)
+        Q.offq_w4a4_linear(ac, asc, aoff, T, N, K, g, wc, wsc, table, out, N)
+    torch.cuda.synchronize()
+    for (wc, wsc, rowsum), out in zip(weights, want):
+        Q.offq_w4a4_linear(ac, asc, aoff, T, N, K, g, wc, wsc, rowsum, out, N)
+        torch.cuda.synchronize()
+    assert Q.offq_get_device_status() == Q.OFFQ_OK
+    for i, out in enumerate(got):
+        assert torch.equal(out, want[i % 4]), i

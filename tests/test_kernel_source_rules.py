@@ -87,3 +87,11 @@ def test_few_token_gemm_reads_early_only_what_its_contract_names():
     head = body[:start]
     assert not re.search(r"first_w\(\)|constants\(\)|__ldg|few_cp_async|p\.(a_\w+|out|w_scale|rowsum)\b", head)
     assert re.search(r"return T <= kEarlyTokens && ", text)
+
+
+def test_kernels_that_finish_weight_tables_do_not_release_their_dependents_early():
+    """At up to 4 tokens offq_w4a4_linear reads codes, scales and row sums before its wait."""
+    for name, kernel in (("quant.cu", "weight_repack_kernel("), ("quant_group.cu", "weight_group_sums_kernel(")):
+        text = source(name)
+        body = block(text, text.index(kernel))
+        assert "griddep_wait();" in body and "griddep_launch_dependents" not in body, kernel
