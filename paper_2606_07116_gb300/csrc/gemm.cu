@@ -856,25 +856,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kT
   if (threadIdx.x == 0 && *abort && p.status != nullptr) atomicExch(p.status, kErrTimeout);
 }
 
-int num_sms() {
-  static int sms[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 template <int OUT, bool kOneBlock, bool kWindows>
 int launch_gemm(const GemmParams& p, cudaStream_t s) {
   auto kern = w4a4_gemm_kernel<OUT, kOneBlock, kWindows>;
   constexpr int kThreads = Roles<kOneBlock>::kThreads;
   constexpr int kSmemBytes = Smem<kOneBlock>::kBytes;
   if (!smem_optin<w4a4_gemm_kernel<OUT, kOneBlock, kWindows>>(kSmemBytes)) return OFFQ_ERR_CUDA;
-  const int sms = num_sms();
+  const int sms = device_sms();
   if (sms < 2) return OFFQ_ERR_CUDA;
   const int tiles = p.m_pairs * p.n_tiles;
   const int clusters = tiles < sms / 2 ? tiles : sms / 2;

@@ -380,18 +380,6 @@ bool reads_early(int64_t T, int64_t K) {
   return T <= kEarlyTokens && (T > 2 ? kEarlyTokens : T) * K <= kEarlyActs;
 }
 
-int few_num_sms() {
-  static int sms[kMaxDevices] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 }  // namespace
 
 namespace offq {
@@ -402,7 +390,7 @@ int few_max_tokens() { return kFewMaxT; }
 int w4a4_linear_few(const uint8_t* a_codes, const float* a_scale, const float* a_offset, int64_t T, int64_t N,
                     int64_t K, int32_t g, const uint8_t* w_codes, const float* w_scale, const float* w_offsum,
                     void* out, int out_dtype, int64_t ldo, int32_t* acc_debug, cudaStream_t stream) {
-  const int sms = few_num_sms();
+  const int sms = device_sms();
   if (sms < 1) return OFFQ_ERR_CUDA;
   FewParams p{};
   p.a_codes = a_codes;

@@ -516,23 +516,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
   if (threadIdx.x == 0 && *abort && p.status != nullptr) atomicExch(p.status, kErrTimeout);
 }
 
-int group_num_sms() {
-  static int sms[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 template <int OUT>
 int launch_group_gemm(const GroupParams& p, cudaStream_t s) {
   auto kern = w4a4_group_gemm_kernel<OUT>;
   if (!smem_optin<w4a4_group_gemm_kernel<OUT>>(kGBytes)) return OFFQ_ERR_CUDA;
-  const int sms = group_num_sms();
+  const int sms = device_sms();
   if (sms < 2) return OFFQ_ERR_CUDA;
   const int tiles = p.m_pairs * p.n_tiles;
   const int clusters = tiles < sms / 2 ? tiles : sms / 2;

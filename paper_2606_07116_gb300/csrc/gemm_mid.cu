@@ -500,18 +500,6 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
   if (threadIdx.x == 0 && *abort && p.status != nullptr) atomicExch(p.status, kErrTimeout);
 }
 
-int mid_num_sms() {
-  static int sms[kMaxDevices] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 // Whether K may be split over S CTAs: at least four k-tiles each, and one wave.
 // Clusters of eight do not fill the chip (1024 x 8192 at 201 tokens, 16 of them:
 // 22.9 us against 11.3 with clusters of four), so they have to fit in two thirds of it.
@@ -557,7 +545,7 @@ namespace offq {
 // 19.5 against 30.2 few-token, 32 x 4096 -> 4096 8.2 against 6.0.
 bool mid_takes(int64_t T, int64_t N, int64_t K, int64_t G) {
   constexpr int64_t kFewTile = 16;
-  const int sms = mid_num_sms();
+  const int sms = device_sms();
   if (sms < 2 || T <= kFewTile) return false;
   const int64_t nk = (K + kMidBK - 1) / kMidBK;
   const int64_t tiles = (N + kMidM - 1) / kMidM * ((T + kMidMaxN - 1) / kMidMaxN);
@@ -580,7 +568,7 @@ bool mid_takes(int64_t T, int64_t N, int64_t K, int64_t G) {
 int w4a4_linear_mid(const uint8_t* a_codes, const float* a_scale, const float* a_offset, int64_t T, int64_t N,
                     int64_t K, int32_t g, const uint8_t* w_codes, const float* w_scale, const float* w_offsum,
                     void* out, int out_dtype, int64_t ldo, int32_t* acc_debug, cudaStream_t stream) {
-  const int sms = mid_num_sms();
+  const int sms = device_sms();
   if (sms < 1) return OFFQ_ERR_CUDA;
   MidParams p{};
   p.a_codes = a_codes;

@@ -574,18 +574,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
   if (threadIdx.x == 0 && *abort && p.status != nullptr) atomicExch(p.status, kErrTimeout);
 }
 
-int mx_num_sms() {
-  static int sms[kMaxDevices] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 // Tiled codes of `blocks` 32-row blocks as [chunk][row block][512 bytes].
 bool encode_codes(CUtensorMap* map, const uint8_t* codes, int64_t blocks, int64_t kchunks, int box_blocks) {
   const auto enc = tensor_map_encoder();
@@ -602,7 +590,7 @@ bool encode_codes(CUtensorMap* map, const uint8_t* codes, int64_t blocks, int64_
 template <int OUT>
 int launch_mx(const CUtensorMap& amap, const CUtensorMap& wmap, const MxGemmParams& p, cudaStream_t s) {
   if (!smem_optin<mx_gemm_kernel<OUT>>(kXSmemMax)) return OFFQ_ERR_CUDA;
-  const int sms = mx_num_sms();
+  const int sms = device_sms();
   if (sms < 2) return OFFQ_ERR_CUDA;
   const int64_t tiles = static_cast<int64_t>(p.m_pairs) * p.n_tiles;
   const int clusters = static_cast<int>(tiles < sms / 2 ? tiles : sms / 2);

@@ -753,25 +753,13 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
   if (tid == 0 && *abort && a.status != nullptr) atomicExch(a.status, kErrTimeout);
 }
 
-int rot_num_sms() {
-  static int sms[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 template <typename Tin, int OUT>
 int launch_rotate(const RotArgs& a, cudaStream_t s) {
   auto kern = rotate_heads_kernel<Tin, OUT>;
   if (!smem_optin<rotate_heads_kernel<Tin, OUT>>(kRotSmem)) return OFFQ_ERR_CUDA;
   // About two CTAs per SM (the shared-memory limit), spread over the heads;
   // each loops over its head's token tiles.
-  const int sms = rot_num_sms();
+  const int sms = device_sms();
   if (sms < 1) return OFFQ_ERR_CUDA;
   const int64_t tiles = (a.T + kTokTile - 1) / kTokTile;
   int64_t per_head = (2 * sms + a.H - 1) / a.H;
@@ -812,7 +800,7 @@ int launch_rotate_mma(const RotArgs& a, cudaStream_t s) {
   }
   // One CTA per SM (shared memory), spread over the heads; each takes every
   // gridDim.x-th of its head's 128-token tiles.
-  const int sms = rot_num_sms();
+  const int sms = device_sms();
   if (sms < 1) return OFFQ_ERR_CUDA;
   const int64_t tiles = (a.T + kTM - 1) / kTM;
   int64_t per_head = sms / a.H > 0 ? sms / a.H : 1;

@@ -59,6 +59,20 @@ inline int launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem
 
 constexpr int kMaxDevices = 64;
 
+// Streaming multiprocessors of the current device, 0 if a query failed. Any thread may call it; the
+// first calls on a device may each ask the runtime.
+inline int device_sms() {
+  static std::atomic<int> cache[kMaxDevices] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+  int sms = dev < kMaxDevices ? cache[dev].load(std::memory_order_relaxed) : 0;
+  if (sms == 0) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev < kMaxDevices) cache[dev].store(sms, std::memory_order_relaxed);
+  }
+  return sms;
+}
+
 // Opts kKernel in to `bytes` of dynamic shared memory on the current device.
 // The attribute belongs to the device's context, so it is set once per device
 // (not once per process): a process that launches on a second GPU sets it

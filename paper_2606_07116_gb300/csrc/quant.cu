@@ -1669,18 +1669,6 @@ int prefer_max_shared(F* kern) {
   return OFFQ_OK;
 }
 
-// Streaming multiprocessors of the current device (queried once per device).
-int sm_count() {
-  static int cache[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (dev < 64 && cache[dev] > 0) return cache[dev];
-  int n = 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (dev < 64) cache[dev] = n;
-  return n;
-}
-
 constexpr int kNoRing = 1;  // launch_ring: use the one-shot kernel instead
 
 // Launches the persistent (ring) form of a row kernel when the input has one
@@ -1692,7 +1680,7 @@ constexpr int kNoRing = 1;  // launch_ring: use the one-shot kernel instead
 template <typename F>
 int launch_ring(F* kern, QuantArgs a, int threads, size_t base_smem, size_t slot_bytes, cudaStream_t stream) {
   if (a.H != 1) return kNoRing;
-  const int sms = sm_count();
+  const int sms = device_sms();
   const int64_t groups = (a.rows + a.rows_per_cta - 1) / a.rows_per_cta;
   if (sms <= 0 || groups <= sms) return kNoRing;
   if (prefer_max_shared(kern) != OFFQ_OK) return OFFQ_ERR_CUDA;
@@ -1791,7 +1779,7 @@ int launch_wide(QuantArgs a, cudaStream_t stream) {
 template <typename Tin>
 int launch_1k(QuantArgs a, cudaStream_t stream) {
   if (a.H != 1 || (a.flags & OFFQ_ROTATE) == 0 || a.G > k1kMaxWarps) return kNoRing;
-  const int sms = sm_count();
+  const int sms = device_sms();
   if (sms <= 0) return OFFQ_ERR_CUDA;
   const int R = std::max(1, 4 / a.G);
   const int64_t groups = (a.rows + R - 1) / R;
@@ -1834,7 +1822,7 @@ template <typename Tin, bool kRot, bool kGen>
 int launch_mx_1k(QuantArgs a, cudaStream_t stream) {
   const int nbw = (a.K + 1023) / 1024;
   if (a.H != 1 || nbw > k1kMaxWarps) return kNoRing;
-  const int sms = sm_count();
+  const int sms = device_sms();
   if (sms <= 0) return OFFQ_ERR_CUDA;
   const int R = std::max(1, 4 / nbw);
   const int64_t groups = (a.rows + R - 1) / R;
@@ -1908,7 +1896,7 @@ int launch_bulk(const QuantArgs& a, cudaStream_t stream) {
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem) != cudaSuccess || per_sm < 1)
     return OFFQ_ERR_CUDA;
-  const int sms = sm_count();
+  const int sms = device_sms();
   if (sms <= 0) return OFFQ_ERR_CUDA;
   const int64_t grid = std::min<int64_t>((a.rows + W - 1) / W, static_cast<int64_t>(sms) * per_sm);
   return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(W * 32), smem, stream, a, S);

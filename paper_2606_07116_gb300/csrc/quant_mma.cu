@@ -577,18 +577,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0 && *abort && a.status != nullptr) atomicExch(a.status, kErrTimeout);
 }
 
-int mma_num_sms() {
-  static int sms[kMaxDevices] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-  if (sms[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = v;
-  }
-  return sms[dev];
-}
-
 }  // namespace
 
 namespace offq {
@@ -598,7 +586,7 @@ int quantize_rows_mma(const MmaQuantRows& p, cudaStream_t stream) {
   if (p.K % 1024 != 0 || p.K < 1024 || p.K / 1024 > kHalfRows) return kNotSuitable;
   if (!p.tiled || !aligned(p.x, 16) || p.ld_t % 8 != 0 || p.ld_t < p.K) return kNotSuitable;
   const int G = p.K / 1024, P = kHalfRows / G;
-  const int sms = mma_num_sms();
+  const int sms = device_sms();
   if (sms < 1) return OFFQ_ERR_CUDA;
   const int64_t tiles = (p.rows + P - 1) / P;
   // Fewer tiles than SMs leave SMs idle: the warp-per-block kernel serves those.

@@ -95,3 +95,18 @@ def test_kernels_that_finish_weight_tables_do_not_release_their_dependents_early
         text = source(name)
         body = block(text, text.index(kernel))
         assert "griddep_wait();" in body and "griddep_launch_dependents" not in body, kernel
+
+
+def test_the_host_keeps_no_plain_mutable_statics():
+    """The ABI's calls may come from several threads at once: what the host code keeps between calls is atomic,
+    under a mutex or set once."""
+    for name in sorted(os.listdir(B.CSRC)):
+        text = source(name)
+        for m in re.finditer(r"^\s+static (?!constexpr|const |_?_?device|__forceinline__|inline|_assert)([^;(]*?)[;={]", text,
+                             flags=re.M):
+            decl = m.group(1)
+            var = decl.split()[-1]
+            synchronised = (re.search(r"std::(atomic|mutex|once_flag)", decl) or f"__atomic_load_n(&{var}" in text
+                            or "std::call_once(once" in text and "std::once_flag once;" in text[m.end():m.end() + 60])
+            assert synchronised, (name, decl)
+    assert sum(source(n).count("cudaDevAttrMultiProcessorCount") for n in os.listdir(B.CSRC)) == 1
