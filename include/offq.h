@@ -110,6 +110,13 @@ enum {
   OFFQ_OFFSET = 2  /* subtract each block's mean as its offset (Eq. 5)        */
 };
 
+/* Forms of offq_w4a4_linear (offq_w4a4_linear_form). */
+enum {
+  OFFQ_FORM_FEW = 1,  /* weights straight into registers, warp-level MMA       */
+  OFFQ_FORM_MID = 2,  /* 128-channel CTAs that split K over a cluster          */
+  OFFQ_FORM_PAIR = 3  /* 256 x 256 tiles of CTA pairs                          */
+};
+
 /*
  * offq_quantize_act -- online activation quantizer (paper Sec. 3.2 Eq. 4-5,
  * Sec. 3 Eq. 1; the online rotation H4 of Sec. 3.3 Step 2 (4)).
@@ -197,6 +204,15 @@ int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, const float* 
                      int64_t T, int64_t N, int64_t K, int32_t g,
                      const uint8_t* w_codes, const float* w_scale, const float* w_offsum,
                      void* out, int out_dtype, int64_t ldo, int32_t* acc_debug, void* stream);
+
+/*
+ * offq_w4a4_linear_form -- the form offq_w4a4_linear takes for a shape on the
+ * current device: OFFQ_FORM_FEW, OFFQ_FORM_MID (K split over a cluster) or
+ * OFFQ_FORM_PAIR; a negative status for a shape it refuses (or, without a
+ * device, OFFQ_ERR_CUDA). A host query, for tests and for labelling
+ * measurements: the results do not depend on the form.
+ */
+int offq_w4a4_linear_form(int64_t T, int64_t N, int64_t K, int32_t g);
 
 /*
  * offq_kv4_quantize -- KV-cache quantizer: offq_quantize_act applied to every

@@ -922,16 +922,36 @@ GemmParams gemm_params(const uint8_t* a_codes, const float* a_scale, const float
   return p;
 }
 
+// The form a shape takes: the cluster form where its cost rule says so, else by tokens.
+int linear_form(int64_t T, int64_t N, int64_t K, int32_t g) {
+  if (mid_takes(T, N, K, K / g)) return OFFQ_FORM_MID;
+  return T <= few_max_tokens() ? OFFQ_FORM_FEW : OFFQ_FORM_PAIR;
+}
+
+// The shape rules of offq_w4a4_linear.
+int check_linear_shape(int64_t T, int64_t N, int64_t K, int32_t g) {
+  if (T < 0 || N < 1 || !is_pow2(g) || g < 32 || g > 8192) return OFFQ_ERR_INVALID_ARG;
+  if (K <= 0 || K % g != 0 || K % 32 != 0) return OFFQ_ERR_INVALID_ARG;
+  if (K > kMaxGemmK || T > 0x3FFFFFFF || N > 0x3FFFFFFF) return OFFQ_ERR_UNSUPPORTED;
+  return OFFQ_OK;
+}
+
 }  // namespace
+
+extern "C" int offq_w4a4_linear_form(int64_t T, int64_t N, int64_t K, int32_t g) {
+  const int rc = check_linear_shape(T, N, K, g);
+  if (rc != OFFQ_OK) return rc;
+  return device_sms() < 1 ? OFFQ_ERR_CUDA : linear_form(T, N, K, g);
+}
 
 extern "C" int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, const float* a_offset, int64_t T,
                                 int64_t N, int64_t K, int32_t g, const uint8_t* w_codes, const float* w_scale,
                                 const float* w_offsum, void* out, int out_dtype, int64_t ldo, int32_t* acc_debug,
                                 void* stream) {
   const int ob = elem_bytes(out_dtype);
-  if (ob == 0 || T < 0 || N < 1 || !is_pow2(g) || g < 32 || g > 8192) return OFFQ_ERR_INVALID_ARG;
-  if (K <= 0 || K % g != 0 || K % 32 != 0 || ldo < N) return OFFQ_ERR_INVALID_ARG;
-  if (K > kMaxGemmK || T > 0x3FFFFFFF || N > 0x3FFFFFFF) return OFFQ_ERR_UNSUPPORTED;
+  const int rc = check_linear_shape(T, N, K, g);
+  if (ob == 0 || ldo < N || rc == OFFQ_ERR_INVALID_ARG) return OFFQ_ERR_INVALID_ARG;
+  if (rc != OFFQ_OK) return rc;
   if (T == 0) return OFFQ_OK;
   if (a_codes == nullptr || a_scale == nullptr || w_codes == nullptr || w_scale == nullptr || w_offsum == nullptr ||
       out == nullptr)
@@ -942,10 +962,11 @@ extern "C" int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, co
     return OFFQ_ERR_MISALIGNED;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (mid_takes(T, N, K, K / g))
+  const int form = linear_form(T, N, K, g);
+  if (form == OFFQ_FORM_MID)
     return w4a4_linear_mid(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype, ldo,
                            acc_debug, s);
-  if (T <= few_max_tokens())
+  if (form == OFFQ_FORM_FEW)
     return w4a4_linear_few(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype, ldo,
                            acc_debug, s);
   const GemmParams p = gemm_params(a_codes, a_scale, a_offset, T, N, K, g, w_codes, w_scale, w_offsum, out, out_dtype,

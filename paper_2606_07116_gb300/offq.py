@@ -30,6 +30,7 @@ OFFQ_ERR_TIMEOUT = -5
 
 OFFQ_F32, OFFQ_BF16, OFFQ_F16 = 0, 1, 2
 OFFQ_ROTATE, OFFQ_OFFSET = 1, 2
+OFFQ_FORM_FEW, OFFQ_FORM_MID, OFFQ_FORM_PAIR = 1, 2, 3
 
 _DTYPE_CODE = {torch.float32: OFFQ_F32, torch.bfloat16: OFFQ_BF16, torch.float16: OFFQ_F16}
 _CODE_DTYPE = {v: k for k, v in _DTYPE_CODE.items()}
@@ -43,6 +44,7 @@ _SIGNATURES = {
     "offq_quantize_act": (_c_int, [_c_vp, _c_int, _c_i64, _c_i64, _c_i64, _c_i32, _c_i32, _c_vp, _c_vp, _c_vp, _c_vp]),
     "offq_w4a4_linear": (_c_int, [_c_vp, _c_vp, _c_vp, _c_i64, _c_i64, _c_i64, _c_i32, _c_vp, _c_vp, _c_vp, _c_vp,
                                   _c_int, _c_i64, _c_vp, _c_vp]),
+    "offq_w4a4_linear_form": (_c_int, [_c_i64, _c_i64, _c_i64, _c_i32]),
     "offq_kv4_quantize": (_c_int, [_c_vp, _c_int, _c_i64, _c_i32, _c_i32, _c_i64, _c_i32, _c_vp, _c_vp, _c_vp, _c_vp]),
     "offq_prepare_weight": (_c_int, [_c_vp, _c_int, _c_i64, _c_i64, _c_i32, _c_i32, _c_vp, _c_vp, _c_vp, _c_vp]),
     "offq_get_device_status": (_c_int, [_c_vp]),
@@ -179,6 +181,14 @@ def offq_w4a4_linear(a_codes: torch.Tensor, a_scale: torch.Tensor, a_offset: Opt
     _check("offq_w4a4_linear", load_library().offq_w4a4_linear(
         _ptr(a_codes), _ptr(a_scale), _ptr(a_offset), T, N, K, g, _ptr(w_codes), _ptr(w_scale),
         _ptr(w_offsum), _ptr(out), _dtype_code(out), ldo, _ptr(acc_debug), _stream(stream)))
+
+
+def offq_w4a4_linear_form(T: int, N: int, K: int, g: int) -> int:
+    """Which of the kernels behind offq_w4a4_linear takes the shape (OFFQ_FORM_*)."""
+    form = load_library().offq_w4a4_linear_form(T, N, K, g)
+    if form < 0:
+        raise OffqError("offq_w4a4_linear_form", form)
+    return form
 
 
 def offq_kv4_quantize(kv: torch.Tensor, T: int, H: int, head_dim: int, ld_token: int, flags: int,

@@ -94,6 +94,17 @@ def test_gemm_argument_checks(lib):
     assert gemm(lib, T=0) == Q.OFFQ_OK
 
 
+def test_linear_form_argument_checks(lib):
+    form = lib.offq_w4a4_linear_form
+    assert form(-1, 64, 1024, 256) == Q.OFFQ_ERR_INVALID_ARG
+    assert form(8, 0, 1024, 256) == Q.OFFQ_ERR_INVALID_ARG
+    assert form(8, 64, 1000, 256) == Q.OFFQ_ERR_INVALID_ARG
+    assert form(8, 64, 1024, 100) == Q.OFFQ_ERR_INVALID_ARG
+    assert form(8, 64, 131072, 4096) == Q.OFFQ_ERR_UNSUPPORTED
+    with pytest.raises(Q.OffqError):
+        Q.offq_w4a4_linear_form(8, 64, 1000, 256)
+
+
 def test_kv_and_weight_argument_checks(lib):
     kv = lib.offq_kv4_quantize
     assert kv(A16, Q.OFFQ_BF16, 4, 0, 128, 128, 3, A16, A16, A16, None) == Q.OFFQ_ERR_INVALID_ARG    # H = 0

@@ -17,6 +17,7 @@ from parity import act_q, check_outputs, epilogue_terms, max_rel_err_floored, we
 pytestmark = pytest.mark.gpu
 
 OUT_DT = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}
+FEW, MID, PAIR = Q.OFFQ_FORM_FEW, Q.OFFQ_FORM_MID, Q.OFFQ_FORM_PAIR
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -118,12 +119,11 @@ def test_oracle_codes_through_gemm():
     (300, 1024, 800, 128, "bf16", None),   # the paper's group size, 8 blocks; several tiles per CTA
     (50, 1024, 258, 256, "bf16", 264),     # N % 4 != 0 with 4 offset blocks (scalar epilogue loads)
     (5, 96, 200, 32, "f32", None),         # K = 96: a k-tile of three 32-channel chunks
-    # 2 x 40 pair tiles: on 76 clusters the 4 tiles past the first wave are cut
-    # along N into 64-column pieces (ragged N at the end), with 4 and 1 offset blocks.
+    # 2 x 40 pair tiles on 76 clusters: a second wave of 4, a ragged last column tile, with 4 and 1 offset blocks.
     (512, 1024, 10200, 256, "bf16", None),
     (512, 1024, 10200, 1024, "f32", 10208),
-    # Decode form (T <= 64): more weight blocks than 4 per SM, so each CTA makes two passes of its
-    # accumulator; and a K that is not a multiple of the 4-k-tile bulk copies.
+    # 9 and 17 tokens: two and four token tiles of the few-token form, more weight blocks than the chip holds
+    # CTAs at once; and 60 chunks of K, the last warps' shares short or empty.
     (9, 1024, 28672, 1024, "bf16", None),
     (17, 1920, 640, 128, "f16", None),
     # Few-token form: one to eight tokens, K = 1056 (33 chunks: the eighths of K are uneven and
@@ -154,6 +154,7 @@ def test_layers(T, K, N, g, out_dt, ldo):
 ])
 def test_few_token_form(T, K, N, g, out_dt):
     """The few-token kernel at the edges of its k-steps, token tiles, offset staging and CTA budgets."""
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == FEW
     ldo = (N + 7) // 8 * 8
     _check_layer(T, K, N, g, out_dt, ldo=ldo, seed=T * 7 + K)
 
@@ -167,12 +168,13 @@ def test_few_token_form(T, K, N, g, out_dt):
     (128, 4096, 264, 4096, "bf16"),  # a whole token tile, K over eight
     (129, 4096, 1024, 1024, "f32"),  # two token tiles of 80: the second starts inside a 32-row block
     (200, 2048, 4096, 32, "bf16"),   # 64 offset blocks
-    (70, 4096, 512, 32, "f32"),      # 128 offset blocks: read from global memory
+    (70, 4096, 512, 32, "f32"),      # 128 offset blocks, the most that the quantizers make: staged past the B stages
     (300, 11008, 4096, 256, "bf16"), # three token tiles of 112
     (48, 512, 8200, 512, "f16"),     # short K: no split; a ragged last channel tile
 ])
 def test_mid_form(T, K, N, g, out_dt):
     """The form between decode and prefill at the edges of its tiles, K splits and offset staging."""
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == MID
     _check_layer(T, K, N, g, out_dt, ldo=(N + 7) // 8 * 8, seed=T + K)
 
 
@@ -216,18 +218,25 @@ def test_accumulator_exact_at_largest_k():
     np.testing.assert_array_equal(y, O.int_gemm(qa, qw).astype(np.float64))
 
 
-@pytest.mark.parametrize("T", [1, 8, 96])
-def test_accumulator_exact_at_maximum_k(T):
-    """K = 65536, the largest the ABI takes, with every code at +-7, through each form of the
-    linear (the few-token form at 1 and 8 tokens, the pair kernel at 96): the largest
-    sum, 15 * 7 * 65536 < 2^24, stays exact."""
-    N, K, g = 256, 65536, 8192
+def _extreme_codes(T, N, K):
+    """Codes of +-7 and a few others; the first rows are all +7, so the largest sum of u q is among their products:
+    15 * 7 * 65536 < 2^24, with either sign."""
     qa = np.full((T, K), 7, dtype=np.int64)
     qa[1::2] = -7
-    qa[:, ::5] = 3
+    qa[2:, ::5] = 3
     qw = np.full((N, K), 7, dtype=np.int64)
-    qw[::3] = -7
-    qw[:, ::7] = 0
+    qw[1::3] = -7
+    qw[2:, ::7] = 0
+    return qa, qw
+
+
+@pytest.mark.parametrize("T,form", [(1, FEW), (8, FEW), (16, FEW), (96, MID)])
+def test_accumulator_exact_at_maximum_k(T, form):
+    """K = 65536, the largest the ABI takes, with every code at +-7, through the few-token form and the one that
+    splits K over a cluster: the largest sum stays exact."""
+    N, K, g = 256, 65536, 8192
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == form
+    qa, qw = _extreme_codes(T, N, K)
     dev = lambda arr, dt: torch.from_numpy(np.ascontiguousarray(arr)).to(dt).cuda()
     sa = np.full(T, 0.5, dtype=np.float32)
     sw = np.full(N, 0.25, dtype=np.float32)
@@ -239,6 +248,51 @@ def test_accumulator_exact_at_maximum_k(T):
                        g, "f32")
     np.testing.assert_array_equal(acc, O.int_gemm(qa + 8, qw))
     np.testing.assert_array_equal(y, 0.125 * O.int_gemm(qa, qw).astype(np.float64))
+
+
+def test_accumulator_exact_at_maximum_k_in_pairs():
+    """K = 65536 through the pair kernel, which sums all of K in one accumulator: 64 rows of each side, repeated to
+    a size that the dispatch gives to it."""
+    T, N, K, g, D = 4096, 2048, 65536, 8192, 64
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == PAIR
+    qa, qw = _extreme_codes(D, D, K)
+    dev = lambda arr, dt: torch.from_numpy(np.ascontiguousarray(arr)).to(dt).cuda()
+    ac = dev(O.tile_codes(O.pack_act_codes(qa)).reshape(-1, K // 2), torch.uint8).repeat(T // D, 1)
+    wc = dev(O.tile_codes(O.pack_weight_codes(qw)).reshape(-1, K // 2), torch.uint8).repeat(N // D, 1)
+    R = dev(qw.reshape(D, K // g, g).sum(axis=2).T, torch.float32).repeat(1, N // D)
+    y = torch.empty((T, N), dtype=torch.float32, device="cuda")
+    acc = torch.zeros((T, N), dtype=torch.int32, device="cuda")
+    Q.offq_w4a4_linear(ac, torch.full((T,), 0.5, device="cuda"), None, T, N, K, g, wc,
+                       torch.full((N,), 0.25, device="cuda"), R, y, N, acc)
+    torch.cuda.synchronize()
+    assert Q.offq_get_device_status() == Q.OFFQ_OK
+    want = dev(O.int_gemm(qa + 8, qw), torch.int32)
+    assert int(want.max()) == -int(want.min()) == 15 * 7 * K
+    assert torch.equal(acc.view(T // D, D, N // D, D), want.view(1, D, 1, D).expand(T // D, D, N // D, D))
+    y_want = dev(0.125 * O.int_gemm(qa, qw).astype(np.float64), torch.float32)
+    assert torch.equal(y.view(T // D, D, N // D, D), y_want.view(1, D, 1, D).expand(T // D, D, N // D, D))
+
+
+@pytest.mark.parametrize("T,K,N,out_dt", [(70, 7296, 512, "f32"), (45, 7328, 520, "bf16")])
+def test_mid_form_reads_constants_from_global_memory(T, K, N, out_dt):
+    """228 and 229 offset blocks of 32 channels, more than the mid form's shared memory holds beside the exchange
+    (row sums alone 117 KB of 200) and more than the library's quantizers make: codes, scales and offsets made here."""
+    g = 32
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == MID
+    rng = np.random.default_rng(T + K)
+    qa, qw = rng.integers(-7, 8, size=(T, K)), rng.integers(-7, 8, size=(N, K))
+    sa, sw = rng.uniform(0.5, 2.0, T).astype(np.float32), rng.uniform(0.01, 0.03, N).astype(np.float32)
+    off = rng.normal(0.0, 3.0, (T, K // g)).astype(np.float32)
+    R = qw.reshape(N, K // g, g).sum(axis=2).T.astype(np.float32)
+    dev = lambda arr, dt: torch.from_numpy(np.ascontiguousarray(arr)).to(dt).cuda()
+    y, acc = _run_gemm(dev(O.tile_codes(O.pack_act_codes(qa)).reshape(-1, K // 2), torch.uint8),
+                       dev(sa, torch.float32), dev(off, torch.float32),
+                       dev(O.tile_codes(O.pack_weight_codes(qw)).reshape(-1, K // 2), torch.uint8),
+                       dev(sw, torch.float32), dev(R, torch.float32), g, out_dt)
+    np.testing.assert_array_equal(acc, O.int_gemm(qa + 8, qw))
+    f64 = [a.astype(np.float64) for a in (sa, off, sw, R)]
+    dot = O.int_gemm(qa, qw)
+    check_outputs(y, O.epilogue(dot, *f64), epilogue_terms(dot, *f64), K // g, out_dt)
 
 
 def test_full_llama2_7b_gate_sampled():
@@ -320,7 +374,7 @@ def test_outputs_near_zero_against_large_row_sums(K, g):
     0, +-1, +-2, ...: every output is a small multiple of s_a s_w next to the 8 s_a R that the
     tensor cores carry in acc'. Removing that term in the integer domain leaves each fp32 output
     within a few rounding errors of the float64 result (max relative error 2e-3 with no floor,
-    f32 out), for one block, 43 blocks, and the unstaged 128-block epilogue."""
+    f32 out), for one block, 43 blocks and 128."""
     T, N = 64, 512
     rng = np.random.default_rng(K + g)
     qa = rng.integers(-7, 8, size=(T, K))
@@ -384,6 +438,7 @@ def test_few_token_forms_agree():
 def test_pair_form_output_routes(T, K, N, g, out_dt, ldo):
     """The 256 x 256 pair kernel's 16-bit rows leave through shared memory, or straight from registers when the
     accumulator is asked for (which the oracle checks): the same bits, and nothing past the N columns."""
+    assert Q.offq_w4a4_linear_form(T, N, K, g) == PAIR
     rows = np.r_[0:3, 127:130, 255:258, T - 2:T]
     y_rows, _, _, w = _check_layer(T, K, N, g, out_dt, seed=T + K, ldo=ldo, rows=rows)
     x = W.activations(T, K, seed=T + K, n_out=2, mult=50.0)
