@@ -1816,8 +1816,11 @@ int launch_1k(QuantArgs a, cudaStream_t stream) {
 }
 
 // quantize_mx_1k_kernel: one row of K/1024 warps per CTA (rows per CTA grow
-// while a CTA has fewer than 4 warps), the ring as launch_1k's. kNoRing when the
-// shape does not fit it (the generic MX kernel serves those).
+// while a CTA has fewer than 4 warps), the ring as launch_1k's. With no more row
+// groups than SMs each CTA takes one, so a ring of one slot does and the runtime is
+// asked nothing: an eager call of one row costs the host 3.1 us (4.2 with the
+// occupancy queries and the attribute on each call). kNoRing when the shape does not
+// fit it (the generic MX kernel serves those).
 template <typename Tin, bool kRot, bool kGen>
 int launch_mx_1k(QuantArgs a, cudaStream_t stream) {
   const int nbw = (a.K + 1023) / 1024;
@@ -1829,14 +1832,15 @@ int launch_mx_1k(QuantArgs a, cudaStream_t stream) {
   if (a.rows + R > 0x7FFFFFFF) return kNoRing;
   auto kern = quantize_mx_1k_kernel<Tin, kRot, kGen>;
   if (prefer_max_shared(kern) != OFFQ_OK) return OFFQ_ERR_CUDA;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxDynSmem)) !=
-      cudaSuccess)
-    return OFFQ_ERR_CUDA;
+  if (!smem_optin<quantize_mx_1k_kernel<Tin, kRot, kGen>>(static_cast<int>(kMaxDynSmem))) return OFFQ_ERR_CUDA;
   const int threads = R * nbw * 32;
   const size_t fixed = kRot ? static_cast<size_t>(R) * nbw * 4096 : 0;
   const size_t slot = static_cast<size_t>(R) * a.K * sizeof(Tin) + 8;
   int best_s = 0, best_per_sm = 0;
-  for (int S = 1; S <= 3; ++S) {
+  if (groups <= sms && fixed + slot <= kMaxDynSmem) {
+    best_s = best_per_sm = 1;
+  }
+  for (int S = 1; S <= 3 && groups > sms; ++S) {
     const size_t smem = fixed + S * slot;
     if (smem > kMaxDynSmem) break;
     int per_sm = 0;
