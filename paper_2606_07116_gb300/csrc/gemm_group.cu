@@ -20,29 +20,39 @@
 // while the MMA fills the other buffers. After a tile's last group the scalers
 // multiply by s_w and store y, rounding once to the output type.
 //
-// What bounds it: the scalers' SM sub-partitions. Per group each has 32 rows x
-// 128 columns to fold (256 cycles of its FMA pipe) and about 280 issue slots of
-// its four scaler warps' waits, loads and bookkeeping, against 296 cycles of MMA
-// (N = 128, A in tensor memory); TMEM reads (64 KB at 900 B/clock) and the three
-// buffers' turnaround fit under that. Hence four warps per sub-partition (the
-// latency of one is three times its issue time), R read while the partial is
-// waited for, s, z and R in shared memory in windows of 16 groups (read from
-// global memory per lane, one row each, they cost 32 cache lines per load), and
-// the registers shifted from the converters to the scalers. The zero-point sits
-// with the scalers' FMAs: subtracting it in the converters costs more issue
-// slots (byte-wise |u - z| and its sign, ~20 operations per 8 codes against 3 for
-// the plain nibbles) and still needs the FMA for a group that does not straddle
-// zero. Measured (per call, weights past the L2; before: eight scaler warps, two
+// What bounds it: issue slots of the SM sub-partitions and the chain of one group.
+// Per group a sub-partition has 32 rows x 128 columns to fold (256 cycles of its
+// FMA pipe) among about 1030 warp instructions (waits, TMEM and shared-memory
+// loads, conversions, bookkeeping: 4120 per CTA), and the kernel takes about 1150
+// cycles per group against 296 of MMA (N = 128, A in tensor memory). Hence four
+// scaler warps per sub-partition (the latency of one is three times its issue
+// time), R read while the partial is waited for, s, z and R in shared memory in
+// windows of 16 groups (read from global memory per lane, one row each, they cost
+// 32 cache lines per load), and the registers shifted from the converters to the
+// scalers. The zero-point sits with the scalers' FMAs: subtracting it in the
+// converters costs more issue slots (byte-wise |u - z| and its sign, ~20 operations
+// per 8 codes against 3 for the plain nibbles) and still needs the FMA for a group
+// that does not straddle zero.
+//
+// At a few groups the time is the chain around them, so: the windows' copies cover
+// only what exists, come from three warps and arrive on their barrier by themselves
+// (one warp that zero-filled the rest and waited for its copies: 64 x 512 -> 512
+// 6.7 us, now 5.5); a tile's channel scales come with its last window (handed round
+// by shuffles, 0.4 us of that); each role reaches its wait for the kernel ahead with
+// its registers and addresses ready (0.2 us).
+//
+// Measured (per call, weights past the L2; before: eight scaler warps, two
 // buffers, z in the operands, s and z by per-lane loads): 2048 x 4096 -> 4096
-// 79.2 us (126.7), -> 11008 195.0 us (314.8), 2048 x 11008 -> 4096 200.2 us
-// (324.0), 1 x 4096 -> 11008 39.2 us (57.2); at 4 groups (64 x 512 -> 512) 6.8 us
-// (6.3), where the launch of twice the warps shows.
+// 75.1 us (126.8), -> 11008 185.9 us (317.4), 2048 x 11008 -> 4096 188.1 us
+// (322.3), 1 x 4096 -> 11008 36.7 us (56.6), 64 x 512 -> 512 5.5 us (6.1), 2048 x
+// 512 -> 8192 32.2 us (34.8). Only at one or two groups does the former still lead:
+// 512 x 128 -> 128 4.9 us (4.0), 2048 x 256 -> 8192 24.4 us (23.2).
 //
 // TMEM (512 columns per CTA): P0, P1, P2 [0, 384), 4 A stages of 32 columns.
 //
 // Warp roles per CTA (32 warps of 64 registers; 48 after the start for warps 0-15, 80 for the scalers):
 //   warp 0       TMEM allocation; in the leader CTA, an elected lane issues the MMAs
-//   warp 1       stages the windows of s, z and R (cp.async)
+//   warps 1-3    stage the windows of s, z and R (cp.async)
 //   warps 4-11   A converters: two per 32-lane TMEM quarter, taking turns by group
 //   warps 12-15  B converters: two per 32-row group (64 rows of B per CTA)
 //   warps 16-31  scalers and epilogue, four per TMEM quarter (32 columns each)
@@ -71,7 +81,7 @@ constexpr int kGroup = GBK;
 constexpr int kGChunks = GBK / 32;  // 16-byte packed chunks per row per k-tile
 constexpr int kGStages = 4;
 constexpr int kGBufs = 3;           // partial buffers
-constexpr int kGRing = 1;           // k-tiles of loads in flight per converter thread (two spill at 64 registers)
+constexpr int kGRing = 1;           // k-tiles of loads in flight per converter thread (two do not fit 64 registers)
 constexpr int kGTurns = 2;          // converter warps per row group, taking turns
 constexpr int kGFirstA = 4, kGFirstB = kGFirstA + 4 * kGTurns;
 constexpr int kGFirstSc = kGFirstB + GBNH / 32 * kGTurns;
@@ -87,13 +97,16 @@ static_assert(kGTurns <= kGStages, "a converter's next stage is at most one ring
 constexpr int kGBStage = GBNH * GBK;  // 8 KB of E4M3 per stage
 constexpr uint32_t kGIdesc = idesc_e4m3_f32(2 * GBM, GBN);  // pair MMA: M = 256, N = 128
 
-// Windows of 16 groups, double-buffered: s and z as [128 rows][16 groups], the
-// four 16-byte pieces of a row at piece ^ (row / 2 % 4), so that eight rows'
-// reads of one piece fall in distinct banks; R as [16 groups][128 columns].
+// Windows of 16 groups, double-buffered: s and z as [128 rows][16 groups], the four
+// 16-byte pieces of a row at piece ^ (row / 2 % 4), so that eight rows' reads of one
+// piece fall in distinct banks; R as [16 groups][128 columns]; a tile's last window
+// with the channel scales.
 constexpr int kGWin = 16;
+constexpr int kGWinThreads = 96;               // warps 1-3
 constexpr int kWinRows = GBM * kGWin * 4;          // 8 KB of s (and of z)
 constexpr int kWinR = kGWin * GBN * 4;             // 8 KB of R
-constexpr int kWinBytes = 2 * kWinRows + kWinR;
+constexpr int kWinW = 2 * kWinRows + kWinR;        // a tile's last window: its channel scales, 512 bytes
+constexpr int kWinBytes = kWinW + GBN * 4;
 
 constexpr int kGOffWin = kGStages * kGBStage;
 constexpr int kGOffBars = kGOffWin + 2 * kWinBytes;
@@ -119,6 +132,7 @@ struct GroupParams {
   int kchunks;  // K / 32
   int vec_sz;   // rows of s and z allow 16-byte copies
   int vec_r;    // rows of R allow 16-byte copies
+  int vec_w;    // s_w too
 };
 
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
@@ -127,8 +141,10 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void sts_zero(uint32_t addr) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(0u) : "memory");
+// Arrives on the mbarrier once all cp.async of this thread so far have landed (the arrival counts against the
+// barrier's initial count).
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
   float2 r;
@@ -180,7 +196,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
       mbar_init(pempty(b), 2 * kGScWarps);
     }
     for (int w = 0; w < 2; ++w) {
-      mbar_init(wfull(w), 1);
+      mbar_init(wfull(w), kGWinThreads);
       mbar_init(wempty(w), kGScWarps);
     }
     *abort = 0;
@@ -194,15 +210,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
   cluster_sync();  // barriers initialised and TMEM allocated in both CTAs
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  griddep_wait();
-  griddep_launch_dependents();
   uint32_t mma_groups = 0;
+  auto start_grid = [] {
+    griddep_wait();
+    griddep_launch_dependents();
+  };
 
   // 16 warps x 48 + 16 warps x 80 = the 32 x 64 registers of the launch.
   if (warp < kGFirstSc) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == 0) {
       // ---------------- MMA issuer (leader CTA) ----------------
+      start_grid();
       // The whole warp runs the loop; an elected lane issues (elect_one).
       if (rank == 0) {
         const uint64_t desc0 = smem_desc_sw128(base);
@@ -236,67 +255,69 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
           }
         }
       }
-    } else if (warp == 1) {
+    } else if (warp < kGFirstA) {
       // ---------------- windows of s, z and R ----------------
+      // Only what exists is copied: rows and columns past the end feed sums that are not stored.
+      const int wt = threadIdx.x - 32;  // of the kGWinThreads that stage
+      start_grid();
       int w = 0, wphase = 0;
       bool ok = true;
       for (int tile = cluster; tile < num_tiles && ok; tile += clusters) {
         const int m0 = (tile / p.n_tiles) * 2 * GBM + static_cast<int>(rank) * GBM;
-        const int n0 = (tile % p.n_tiles) * GBN;
+        const int n = (tile % p.n_tiles) * GBN + 4 * lane;
+        const int rows = p.T - m0 < GBM ? p.T - m0 : GBM;  // may be negative
         for (int k0 = 0; k0 < nk; k0 += kGWin) {
           ok = __all_sync(0xFFFFFFFFu, wait_cluster(wempty(w), wphase ^ 1, abort));
           if (!ok) break;
           const uint32_t wb = base + kGOffWin + w * kWinBytes;
-          // Lane l copies piece l % 4 (groups 4 (l % 4) ..) of rows l / 4, l / 4 + 8, ...
-          const int g = (lane & 3) * 4;
-          for (int r = lane >> 2; r < GBM; r += 8) {
-            const int t = m0 + r;
-            const int64_t src = static_cast<int64_t>(t) * nk + k0 + g;
+          const int ng = nk - k0 < kGWin ? nk - k0 : kGWin;
+          const int pieces = (ng + 3) / 4;  // of four groups per row: 1 to 4, which divide kGWinThreads
+          const int g = wt % pieces * 4;
+          for (int r = wt / pieces; r < rows; r += kGWinThreads / pieces) {
+            const int64_t src = static_cast<int64_t>(m0 + r) * nk + k0 + g;
             const uint32_t dst = wb + win_off(r, g);
-            if (p.vec_sz) {
-              if (t < p.T && k0 + g < nk) {  // nk % 4 == 0: pieces are whole
-                cp_async16(dst, p.a_scale + src);
-                cp_async16(dst + kWinRows, p.a_zero + src);
-              } else {
-                sts128(dst, 0u, 0u, 0u, 0u);
-                sts128(dst + kWinRows, 0u, 0u, 0u, 0u);
-              }
+            if (p.vec_sz) {  // nk % 4 == 0: pieces are whole
+              cp_async16(dst, p.a_scale + src);
+              cp_async16(dst + kWinRows, p.a_zero + src);
             } else {
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
-                if (t < p.T && k0 + g + i < nk) {
+                if (g + i < ng) {
                   cp_async4(dst + 4 * i, p.a_scale + src + i);
                   cp_async4(dst + kWinRows + 4 * i, p.a_zero + src + i);
-                } else {
-                  sts_zero(dst + 4 * i);
-                  sts_zero(dst + kWinRows + 4 * i);
                 }
               }
             }
           }
-          const int n = n0 + 4 * lane;
-          for (int i = 0; i < kGWin && k0 + i < nk; ++i) {
+          for (int i = warp - 1; i < ng; i += kGWinThreads / 32) {
             const float* src = p.gsum + static_cast<int64_t>(k0 + i) * p.N + n;
             const uint32_t dst = wb + 2 * kWinRows + i * GBN * 4 + lane * 16;
-            if (p.vec_r && n < p.N) {  // N % 4 == 0: whole pieces
-              cp_async16(dst, src);
+            if (p.vec_r) {  // N % 4 == 0: whole pieces
+              if (n < p.N) cp_async16(dst, src);
             } else {
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                if (n + q < p.N)
-                  cp_async4(dst + 4 * q, src + q);
-                else
-                  sts_zero(dst + 4 * q);
-              }
+              for (int q = 0; q < 4; ++q)
+                if (n + q < p.N) cp_async4(dst + 4 * q, src + q);
             }
           }
-          asm volatile("cp.async.wait_all;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(wfull(w));
+          if (k0 + kGWin >= nk && warp == 1) {
+            const float* src = p.w_scale + n;
+            const uint32_t dst = wb + kWinW + lane * 16;
+            if (p.vec_w) {
+              if (n < p.N) cp_async16(dst, src);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (n + q < p.N) cp_async4(dst + 4 * q, src + q);
+            }
+          }
+          // Arrives when this thread's copies have landed: the next window's are issued meanwhile.
+          cp_async_arrive(wfull(w));
           w ^= 1;
           if (w == 0) wphase ^= 1;
         }
       }
+      asm volatile("cp.async.wait_all;" ::: "memory");  // after an abort too, no copy outlives the CTA
     } else if (warp >= kGFirstA && warp < kGFirstSc) {
       // ---------------- converters: packed codes -> E4M3 operands ----------------
       // Two warps per 32-row group take turns by group, each with kGRing of its
@@ -333,6 +354,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
           new_tile();
       };
       new_tile();
+      start_grid();
       // This warp's groups: every kGTurns-th of all tiles' groups.
       const int my_tiles = cluster < num_tiles ? (num_tiles - cluster + clusters - 1) / clusters : 0;
       int64_t left = (static_cast<int64_t>(my_tiles) * nk - turn + kGTurns - 1) / kGTurns;
@@ -406,14 +428,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
     const uint32_t pempty_l = leader_addr(pempty(0));
     int b = 0, bphase = 0, w = 0, wphase = 0;
     bool ok = true;
+    start_grid();
     for (int tile = cluster; tile < num_tiles && ok; tile += clusters) {
       const int m0 = (tile / p.n_tiles) * 2 * GBM + static_cast<int>(rank) * GBM;
       const int t = m0 + rl;
       const int n0 = (tile % p.n_tiles) * GBN + c0;
       const bool warp_on = m0 + quarter * 32 < p.T && n0 < p.N;  // else nothing of this warp's is written
-      // Channel scale of column c0 + lane, handed round at the tile's end.
-      static_assert(kGScCols == 32, "one channel scale per lane");
-      const float ws = n0 + lane < p.N ? __ldg(p.w_scale + n0 + lane) : 0.f;
       uint64_t S2[kGScCols / 2];  // running sums of this row's columns c0 .. c0 + kGScCols, packed in pairs
 #pragma unroll
       for (int i = 0; i < kGScCols / 2; ++i) S2[i] = 0ull;
@@ -479,6 +499,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
           }
         }
         if (!ok) break;
+        if (k0 + kGWin >= nk) {
+          // The tile's last window carries its channel scales.
+          const float4* wrow = reinterpret_cast<const float4*>(smem + kGOffWin + w * kWinBytes + kWinW + c0 * 4);
+#pragma unroll
+          for (int q = 0; q < kGScCols / 4; ++q) {
+            const float4 wv = wrow[q];
+            S2[2 * q] = mul2v(pack2(wv.x, wv.y), S2[2 * q]);
+            S2[2 * q + 1] = mul2v(pack2(wv.z, wv.w), S2[2 * q + 1]);
+          }
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(wempty(w));
         w ^= 1;
@@ -489,10 +519,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
         for (int c = 0; c < kGScCols; c += 8) {
           float y[8];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float w0 = __shfl_sync(0xFFFFFFFFu, ws, c + 2 * i), w1 = __shfl_sync(0xFFFFFFFFu, ws, c + 2 * i + 1);
-            unpack2(mul2v(pack2(w0, w1), S2[c / 2 + i]), y[2 * i], y[2 * i + 1]);
-          }
+          for (int i = 0; i < 4; ++i) unpack2(S2[c / 2 + i], y[2 * i], y[2 * i + 1]);
           const int nvalid = p.N - n0 - c < 8 ? p.N - n0 - c : 8;
           if (t < p.T && nvalid > 0) store_out<OUT, 8>(p.out, static_cast<int64_t>(t) * p.ldo + n0 + c, y, nvalid);
         }
@@ -566,6 +593,7 @@ extern "C" int offq_w4a4_linear_group(const uint8_t* a_codes, const float* a_sca
   p.kchunks = static_cast<int>(K / 32);
   p.vec_sz = p.Gq % 4 == 0 && aligned(a_scale, 16) && aligned(a_zero, 16);
   p.vec_r = N % 4 == 0 && aligned(w_groupsum, 16);
+  p.vec_w = N % 4 == 0 && aligned(w_scale, 16);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   switch (out_dtype) {
     case OFFQ_F32: return launch_group_gemm<OFFQ_F32>(p, s);

@@ -244,3 +244,26 @@ def test_group_sums_feed_the_linear_behind_them(T):
     assert Q.offq_get_device_status() == Q.OFFQ_OK
     for i, out in enumerate(got):
         assert torch.equal(out, want[i % 4]), i
+
+
+@pytest.mark.parametrize("T,K,N", [(37, 512, 136), (130, 2304, 264)])
+def test_group_gemm_tables_off_alignment(T, K, N):
+    """s, z, R and the channel scales at 4-byte aligned addresses that allow no 16-byte copies: the same bits."""
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    x = (torch.randn((T, K), generator=gen, device="cuda") * 3).to(torch.bfloat16)
+    wc, wsc, _ = Q.prepare_weight(torch.randn((N, K), generator=gen, device="cuda") * 0.02, 128, rotate=False)
+    R = Q.weight_group_sums(wc, N, K)
+    ac, s, z = Q.quantize_act_group(x, 128, rotate=False)
+    shifted = []
+    for t in (s, z, wsc, R):
+        buf = torch.empty(t.numel() + 1, device="cuda")
+        buf[1:] = t.reshape(-1)
+        shifted.append(buf[1:])
+        assert shifted[-1].data_ptr() % 16 == 4
+    outs = [torch.empty((T, N), device="cuda") for _ in range(2)]
+    Q.offq_w4a4_linear_group(ac, s, z, T, N, K, 128, wc, wsc, R, outs[0], N)
+    s1, z1, w1, R1 = shifted
+    Q.offq_w4a4_linear_group(ac, s1, z1, T, N, K, 128, wc, w1, R1, outs[1], N)
+    torch.cuda.synchronize()
+    assert Q.offq_get_device_status() == Q.OFFQ_OK
+    assert torch.equal(outs[0], outs[1])
