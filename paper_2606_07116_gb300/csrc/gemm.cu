@@ -87,7 +87,7 @@ constexpr int kACol0 = kAccCols;   // A operand stages live in TMEM after the ac
 constexpr int kAColsPerStage = BK / 4;  // 4 E4M3 values per 32-bit column
 constexpr int kTmemCols = 512;
 static_assert(kACol0 + Roles<true>::kStages * kAColsPerStage <= kTmemCols, "TMEM budget");
-// Several offset blocks: the correction sum_b (o_b - 8 s_a) R[b][n] of a tile is
+// Several offset blocks: the correction sum_b o_b R[b][n] of a tile is
 // computed while its MMAs run; accumulator columns 0..127 keep theirs in TMEM
 // after the A stages, columns 128..255 in shared memory.
 constexpr int kCorrCol0 = kACol0 + Roles<false>::kStages * kAColsPerStage;
@@ -225,10 +225,6 @@ __device__ __forceinline__ uint64_t lds64(uint32_t addr) {
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-template <int kBytes>
-__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(kBytes) : "memory");
-}
 template <int OUT>
 __device__ __forceinline__ uint32_t pack_out(float a, float b) {
   if (OUT == OFFQ_BF16) {
@@ -261,6 +257,7 @@ __device__ __forceinline__ int b_block(const GemmParams& p, int tile, uint32_t r
 // runs its own instantiation, so the register allocation of the common one-block
 // kernel does not carry the G-term epilogue loop, nor that of up to kMaxStageG
 // blocks the reload of a window's sums (6912 -> 2560, 27 blocks: 50 us, 56 with it).
+// All have 80 registers; with windows two of the three output types spill 4 to 12 bytes.
 template <int OUT, bool kOneBlock, bool kWindows>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<kOneBlock>::kThreads, 1)
     w4a4_gemm_kernel(const GemmParams p) {

@@ -112,12 +112,6 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int j) {
   return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w;
 }
 
-__device__ __forceinline__ void few_cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void few_cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
 __device__ __forceinline__ void few_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // NT: 8-token tiles per CTA (and warp); kFewWarps warps split K. CTAS: CTAs per
@@ -185,7 +179,7 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
       for (int i = threadIdx.x; i < p.G * 32; i += KS * 32) {
         const int nn = rb * 32 + (i & 31);
         if (nn < p.N)
-          few_cp_async4(smem_u32(sR + i), p.rowsum + static_cast<int64_t>(i >> 5) * p.N + nn);
+          cp_async<4>(smem_u32(sR + i), p.rowsum + static_cast<int64_t>(i >> 5) * p.N + nn);
         else
           sR[i] = 0.f;
       }
@@ -213,7 +207,7 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
         const int piece = lane + 32 * i, c = piece / F::kTokens, r = piece % F::kTokens;
         const uint32_t dst = ring + (slot * 4 + c) * F::kChunkPitch + r * 16;
         if (4 * s + c < kc)
-          few_cp_async16(dst, p.a_codes + static_cast<uint32_t>(4 * s + c) * 512u + r * 16);
+          cp_async<16>(dst, p.a_codes + static_cast<uint32_t>(4 * s + c) * 512u + r * 16);
         else
           sts128(dst, 0u, 0u, 0u, 0u);
       }
@@ -226,7 +220,7 @@ __global__ void __launch_bounds__(kFewWarps * 32, CTAS) w4a4_few_kernel(const Fe
   if (p.staged && p.a_offset != nullptr) {
     const int cnt = p.T * p.G;
     for (int i = threadIdx.x; i < cnt; i += KS * 32)
-      few_cp_async4(smem_u32(sO + i), p.a_offset + i);
+      cp_async<4>(smem_u32(sO + i), p.a_offset + i);
   }
   // Scales of the tokens this warp finishes: lane i holds token ks + KS i.
   const int my_tok = ks + KS * lane;

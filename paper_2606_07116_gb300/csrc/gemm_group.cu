@@ -50,7 +50,8 @@
 //
 // TMEM (512 columns per CTA): P0, P1, P2 [0, 384), 4 A stages of 32 columns.
 //
-// Warp roles per CTA (32 warps of 64 registers; 48 after the start for warps 0-15, 80 for the scalers):
+// Warp roles per CTA (32 warps of 64 registers, with 56 / 92 bytes of spill stores / loads; 48 after the start for
+// warps 0-15, 80 for the scalers):
 //   warp 0       TMEM allocation; in the leader CTA, an elected lane issues the MMAs
 //   warps 1-3    stage the windows of s, z and R (cp.async)
 //   warps 4-11   A converters: two per 32-lane TMEM quarter, taking turns by group
@@ -135,12 +136,6 @@ struct GroupParams {
   int vec_w;    // s_w too
 };
 
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 // Arrives on the mbarrier once all cp.async of this thread so far have landed (the arrival counts against the
 // barrier's initial count).
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
@@ -277,14 +272,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
             const int64_t src = static_cast<int64_t>(m0 + r) * nk + k0 + g;
             const uint32_t dst = wb + win_off(r, g);
             if (p.vec_sz) {  // nk % 4 == 0: pieces are whole
-              cp_async16(dst, p.a_scale + src);
-              cp_async16(dst + kWinRows, p.a_zero + src);
+              cp_async<16>(dst, p.a_scale + src);
+              cp_async<16>(dst + kWinRows, p.a_zero + src);
             } else {
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
                 if (g + i < ng) {
-                  cp_async4(dst + 4 * i, p.a_scale + src + i);
-                  cp_async4(dst + kWinRows + 4 * i, p.a_zero + src + i);
+                  cp_async<4>(dst + 4 * i, p.a_scale + src + i);
+                  cp_async<4>(dst + kWinRows + 4 * i, p.a_zero + src + i);
                 }
               }
             }
@@ -293,22 +288,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
             const float* src = p.gsum + static_cast<int64_t>(k0 + i) * p.N + n;
             const uint32_t dst = wb + 2 * kWinRows + i * GBN * 4 + lane * 16;
             if (p.vec_r) {  // N % 4 == 0: whole pieces
-              if (n < p.N) cp_async16(dst, src);
+              if (n < p.N) cp_async<16>(dst, src);
             } else {
 #pragma unroll
               for (int q = 0; q < 4; ++q)
-                if (n + q < p.N) cp_async4(dst + 4 * q, src + q);
+                if (n + q < p.N) cp_async<4>(dst + 4 * q, src + q);
             }
           }
           if (k0 + kGWin >= nk && warp == 1) {
             const float* src = p.w_scale + n;
             const uint32_t dst = wb + kWinW + lane * 16;
             if (p.vec_w) {
-              if (n < p.N) cp_async16(dst, src);
+              if (n < p.N) cp_async<16>(dst, src);
             } else {
 #pragma unroll
               for (int q = 0; q < 4; ++q)
-                if (n + q < p.N) cp_async4(dst + 4 * q, src + q);
+                if (n + q < p.N) cp_async<4>(dst + 4 * q, src + q);
             }
           }
           // Arrives when this thread's copies have landed: the next window's are issued meanwhile.

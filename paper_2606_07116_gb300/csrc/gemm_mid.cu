@@ -92,10 +92,6 @@ struct MidParams {
   int off_o;               // staged offsets, within the B stages' space
 };
 
-__device__ __forceinline__ void mid_cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
 // D[tmem] (+)= A[tmem] * B[smem]^T, one CTA, E4M3 operands, fp32 accumulate.
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                        uint32_t accumulate) {
@@ -200,7 +196,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
   for (int i = threadIdx.x; i < (ch1 - ch0) * kMidChunk; i += kMidThreads) {
     const int tok = t0 + ch0 * kMidChunk + i;
     if (tok < p.T)
-      mid_cp_async4(smem_u32(sSa + i), p.a_scale + tok);
+      cp_async<4>(smem_u32(sSa + i), p.a_scale + tok);
     else
       sSa[i] = 0.f;
   }
@@ -326,7 +322,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
     for (int i = threadIdx.x; i < p.G * kMidM; i += kMidThreads) {
       const int n = n0 + (i & (kMidM - 1));
       if (n < p.N)
-        mid_cp_async4(base + i * 4, p.rowsum + static_cast<int64_t>(i / kMidM) * p.N + n);
+        cp_async<4>(base + i * 4, p.rowsum + static_cast<int64_t>(i / kMidM) * p.N + n);
       else
         *reinterpret_cast<float*>(smem + i * 4) = 0.f;
     }
@@ -336,7 +332,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) w4a4_mid_kernel(const MidParam
       const int cnt = (left < own ? left : own) * p.G;  // may be negative
       for (int i = threadIdx.x; i < cnt; i += kMidThreads) {
         const int r = i / p.G, b = i - r * p.G;
-        mid_cp_async4(base + p.off_o + (r * p.gp + b) * 4, p.a_offset + static_cast<int64_t>(own_t0) * p.G + i);
+        cp_async<4>(base + p.off_o + (r * p.gp + b) * 4, p.a_offset + static_cast<int64_t>(own_t0) * p.G + i);
       }
     }
   }

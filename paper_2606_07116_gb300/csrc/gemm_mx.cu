@@ -148,10 +148,6 @@ __device__ __forceinline__ void tmem_st_2cols(uint32_t taddr, const uint32_t* r)
   asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(taddr), "r"(r[0]), "r"(r[1]) : "memory");
 }
 
-__device__ __forceinline__ void mx_cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
 // Pair tile index -> (m-pair, n-tile), in raster groups of m-pairs (as the pair
 // kernel of gemm.cu: a weight tile is read from DRAM about once per group).
 __device__ __forceinline__ void mx_tile(const MxGemmParams& p, int tile, int& mp, int& nt) {
@@ -389,7 +385,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
       // The tile's constants, while its MMAs run (asynchronous copies: their latencies overlap).
       auto stage = [](float* dst, const float* src, bool exists) {
         if (exists)
-          mx_cp_async4(smem_u32(dst), src);
+          cp_async<4>(smem_u32(dst), src);
         else
           *dst = 0.f;
       };

@@ -29,11 +29,6 @@ inline int elem_bytes(int dtype) {
   }
 }
 
-inline int launch_status() {
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? OFFQ_OK : OFFQ_ERR_CUDA;
-}
-
 // Launches kern<<<grid, block, smem, stream>>>(args...) with programmatic
 // stream serialization: the kernel may be scheduled while the previous kernel
 // in the stream finishes, and waits for it (griddepcontrol.wait) before it

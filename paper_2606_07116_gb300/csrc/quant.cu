@@ -1001,7 +1001,8 @@ __global__ void __launch_bounds__(k1kMaxWarps * 32, 1) quantize_rows_1k_kernel(c
 // barrier and two integer divisions per butterfly took, against this form:
 // 1 x 4096 (no rotation) 17.2 us against 2.0, 64 x 11008 (g = 256, rotated) 24.4
 // against 5.5, 2048 x 11008 159 against 42.5, 1000 x 8192 fp32 (g = 8192) 81.9
-// against 25.3. The whole-span instantiation keeps prefill widths (4096 x 14336,
+// against 25.3. The rotating general instantiation spills 76 / 72 bytes at the 72
+// registers that 28 warps leave. The whole-span instantiation keeps prefill widths (4096 x 14336,
 // g = 1024: 52.8 us either way before; the general one adds the normalisation and
 // the runtime stages to every span).
 

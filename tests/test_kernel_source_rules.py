@@ -85,7 +85,7 @@ def test_few_token_gemm_reads_early_only_what_its_contract_names():
     assert "first_w();" in after and not re.search(r"first_w\(\)|constants\(\)|__ldg|cp_async|p\.a_|p\.out", before)
     assert before.count(";") == 1 and "prefetch_w();" in before
     head = body[:start]
-    assert not re.search(r"first_w\(\)|constants\(\)|__ldg|few_cp_async|p\.(a_\w+|out|w_scale|rowsum)\b", head)
+    assert not re.search(r"first_w\(\)|constants\(\)|__ldg|cp_async<|p\.(a_\w+|out|w_scale|rowsum)\b", head)
     assert re.search(r"return T <= kEarlyTokens && ", text)
 
 
