@@ -751,7 +751,8 @@ def time_decode(device, args, flush_l2, stream):
     if st != Q.OFFQ_OK:
         raise RuntimeError(f"device status after the decode sweep: {Q.status_string(st)}")
     del sets
-    kern = "w4a4_few_kernel (T <= 16)" if best["T"] <= 16 else "w4a4_mid_kernel (tcgen05, 16 < T)"
+    kern = {Q.OFFQ_FORM_FEW: "w4a4_few_kernel", Q.OFFQ_FORM_MID: "w4a4_mid_kernel",
+            Q.OFFQ_FORM_PAIR: "w4a4_gemm_kernel"}[Q.offq_w4a4_linear_form(best["T"], N, K, g)]
     out["roofline"] = {"bound": "hbm", "kernel": f"{kern} weight stream (T = {best['T']})",
                        "achieved": best["weight_gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
                        "frac": best["weight_frac"], "bytes": w_bytes}
@@ -759,19 +760,49 @@ def time_decode(device, args, flush_l2, stream):
 
 
 def time_gemm_shape(device, args, flush_l2, stream):
-    """One offq_w4a4_linear shape alone (T, K -> N, block g; codes made without
-    the rotation unless g < K), per-call events after an L2 flush: a side
-    measurement for profiling, not the bench line."""
+    """One linear's GEMM alone (T, K -> N, block g; codes made without the rotation unless g < K), per-call
+    events after an L2 flush: a side measurement for profiling, not the bench line. --gemm T,K,N[,path] with
+    path token (offq_w4a4_linear, the default), group (offq_w4a4_linear_group) or mx (offq_mx_linear)."""
     import torch
     from paper_2606_07116_gb300 import offq as Q
-    T, K, N = (int(v) for v in args.gemm.split(",")[:3])
+    spec = args.gemm.split(",")
+    T, K, N = (int(v) for v in spec[:3])
+    path = spec[3] if len(spec) > 3 else "token"
     g = W.block_for(K)
+    rot = g < K and not (path == "group" and g > 512)
     w = workload_by_name(args.workload)
     x = device_activations(T, K, w, seed=900, device=device)
-    codes, scale, off = Q.quantize_act(x, g, rotate=g < K, offset=True)
-    del x
-    wc, ws, wr = Q.prepare_weight(device_weights(N, K, seed=901, device=device), g, rotate=g < K)
+    wt = device_weights(N, K, seed=901, device=device)
     y = torch.empty((T, N), dtype=torch.bfloat16, device=device)
+    if path == "token":
+        kern = {Q.OFFQ_FORM_FEW: "w4a4_few_kernel", Q.OFFQ_FORM_MID: "w4a4_mid_kernel",
+                Q.OFFQ_FORM_PAIR: "w4a4_gemm_kernel"}[Q.offq_w4a4_linear_form(T, N, K, g)]
+        codes, scale, off = Q.quantize_act(x, g, rotate=rot, offset=True)
+        wc, ws, wr = Q.prepare_weight(wt, g, rotate=rot)
+        peak_x = FP8_PER_BF16
+
+        def call():
+            Q.offq_w4a4_linear(codes, scale, off, T, N, K, g, wc, ws, wr, y, N, None, stream)
+    elif path == "group":
+        kern = "w4a4_group_gemm_kernel"
+        codes, scale, zero = Q.quantize_act_group(x, g, rotate=rot)
+        wc, ws, _ = Q.prepare_weight(wt, g, rotate=rot)
+        wr = Q.weight_group_sums(wc, N, K)
+        peak_x = FP8_PER_BF16
+
+        def call():
+            Q.offq_w4a4_linear_group(codes, scale, zero, T, N, K, 128, wc, ws, wr, y, N, stream)
+    elif path == "mx":
+        kern = "mx_gemm_kernel"
+        codes, shifts, scale, off = Q.quantize_act_mx(x, g, rotate=rot, offset=True)
+        wc, wsh, ws, wr = Q.prepare_weight_mx(wt, g, rotate=rot)
+        peak_x = 3.0 * FP8_PER_BF16
+
+        def call():
+            Q.offq_mx_linear(codes, shifts, scale, off, T, N, K, g, wc, wsh, ws, wr, y, N, stream)
+    else:
+        raise SystemExit(f"--gemm: unknown path {path}")
+    del x, wt
     reps = max(1, min(args.steps, 50))
     ts = []
     for r in range(args.warmup + reps):
@@ -779,7 +810,7 @@ def time_gemm_shape(device, args, flush_l2, stream):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record(stream)
-        Q.offq_w4a4_linear(codes, scale, off, T, N, K, g, wc, ws, wr, y, N, None, stream)
+        call()
         e1.record(stream)
         torch.cuda.synchronize(device)
         if r >= args.warmup:
@@ -790,9 +821,9 @@ def time_gemm_shape(device, args, flush_l2, stream):
     ms = sum(ts) / len(ts)
     peaks = load_peaks()
     tflops = 2.0 * T * N * K / (ms * 1e-3) / 1e12
-    peak = peaks["bf16_tflops"] * FP8_PER_BF16
-    return {"gemm": {"T": T, "K": K, "N": N, "g": g}, "us": round(ms * 1e3, 2), "tflops": round(tflops, 1),
-            "peak": peak, "frac": round(tflops / peak, 4), "reps": reps}
+    peak = peaks["bf16_tflops"] * peak_x
+    return {"gemm": {"T": T, "K": K, "N": N, "g": g, "path": path, "kernel": kern}, "us": round(ms * 1e3, 2),
+            "tflops": round(tflops, 1), "peak": peak, "frac": round(tflops / peak, 4), "reps": reps}
 
 
 def _pair_times(events):
@@ -1132,8 +1163,8 @@ def main():
     ap.add_argument("--decode", action="store_true",
                     help="time only the decode sweep (1/8/32/64 tokens) and print that object")
     ap.add_argument("--gemm", default="",
-                    help="T,K,N: time only offq_w4a4_linear at this shape (bf16 out) and print that object "
-                         "(a side measurement for profiling, not the bench line)")
+                    help="T,K,N[,path]: time only one linear's GEMM at this shape (bf16 out; path token, group or mx) "
+                         "and print that object (a side measurement for profiling, not the bench line)")
     ap.add_argument("--quant-sites", action="store_true",
                     help="time only the activation quantizer on the larger prefill inputs and print that object "
                          "(a side measurement for profiling, not the bench line)")
