@@ -57,3 +57,15 @@ def test_seeded_and_distinct_per_seed():
     c = bench.device_activations(64, 512, w, seed=8, device=CPU)
     assert torch.equal(a, b)
     assert not torch.equal(a, c)
+
+
+def test_traffic_record_is_in_the_tree_and_read_for_its_sources():
+    """The ncu record behind the line's `traffic`: complete, consistent, and used only for the sources it names."""
+    import json
+    with open(os.path.join(ROOT, "profiles", "gemm_traffic.json")) as f:
+        rec = json.load(f)
+    per = rec["per_launch"]
+    assert len(per) == len(bench.workload_by_name("llama2_70b").layers)
+    assert rec["bytes_per_launch"] == sum(p["dram_read"] + p["dram_write"] for p in per) // len(per)
+    want = rec if rec["gemm_src_sha256"] == bench.gemm_source_digest() else None
+    assert bench.load_traffic_record() == want
