@@ -132,7 +132,8 @@ enum {
  *   x       device, [T][ldx] elements of x_dtype (OFFQ_F32/BF16/F16), row-major;
  *           16-byte aligned, ldx * sizeof(elem) a multiple of 16, ldx >= K.
  *   T       token rows, >= 0 (T = 0 launches nothing).
- *   K       channels, a multiple of g and of 32, K <= 32768.
+ *   K       channels, a multiple of g and of 32, K <= 32768 and K <= 128 g
+ *           (more offset blocks per row: OFFQ_ERR_UNSUPPORTED).
  *   g       block size, power of two in [32, 8192].
  *   flags   OR of OFFQ_ROTATE, OFFQ_OFFSET.
  *   codes   device, offq_act_codes_bytes(T, K) bytes, activation code format in
@@ -247,7 +248,8 @@ int offq_kv4_quantize(const void* kv, int dtype, int64_t T, int32_t H, int32_t h
  *   R[b][n] = sum_{k in block b} q_w[n][k]   (integers, stored as float32)
  *
  *   w         device, [N][K] of dtype, row-major, 16-byte aligned.
- *   N, K, g   as in offq_w4a4_linear.
+ *   N         output channels, N >= 1.
+ *   K, g      as in offq_quantize_act (K <= 128 g too).
  *   rotate    nonzero to fuse the block Hadamard.
  *   w_codes   device, offq_weight_codes_bytes(N, K) bytes, weight code format in
  *             the tiled operand layout (padding rows set to zero), 16-B aligned.
