@@ -199,7 +199,7 @@ int offq_quantize_act(const void* x, int x_dtype, int64_t T, int64_t K, int64_t 
  * ahead of it in the stream has finished (programmatic dependent launch), so
  * they must not be written by a kernel that releases its dependents early
  * (ordinary kernels never do; nor does any kernel of this library that finishes
- * a table of the weights). With more tokens nothing is read that early.
+ * one of these three). With more tokens nothing is read that early.
  */
 int offq_w4a4_linear(const uint8_t* a_codes, const float* a_scale, const float* a_offset,
                      int64_t T, int64_t N, int64_t K, int32_t g,
