@@ -225,15 +225,6 @@ __device__ __forceinline__ uint64_t lds64(uint32_t addr) {
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-template <int OUT>
-__device__ __forceinline__ uint32_t pack_out(float a, float b) {
-  if (OUT == OFFQ_BF16) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&v);
-  }
-  const __half2 v = __floats2half2_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
 
 // Row block (of 32 rows) of this CTA's A rows / B rows for a pair tile.
 __device__ __forceinline__ int a_block(const GemmParams& p, int tile, uint32_t rank, int quarter) {

@@ -39,18 +39,19 @@
 // (one warp that zero-filled the rest and waited for its copies: 64 x 512 -> 512
 // 6.7 us, now 5.5); a tile's channel scales come with its last window (handed round
 // by shuffles, 0.4 us of that); each role reaches its wait for the kernel ahead with
-// its registers and addresses ready (0.2 us).
+// its registers and addresses ready (0.2 us); outputs leave in whole 64-byte runs.
 //
 // Measured (per call, weights past the L2; before: eight scaler warps, two
 // buffers, z in the operands, s and z by per-lane loads): 2048 x 4096 -> 4096
-// 75.1 us (126.8), -> 11008 185.9 us (317.4), 2048 x 11008 -> 4096 188.1 us
-// (322.3), 1 x 4096 -> 11008 36.7 us (56.6), 64 x 512 -> 512 5.5 us (6.1), 2048 x
-// 512 -> 8192 32.2 us (34.8). Only at one or two groups does the former still lead:
-// 512 x 128 -> 128 4.9 us (4.0), 2048 x 256 -> 8192 24.4 us (23.2).
+// 72.4 us (126.8), -> 11008 175.8 us (315.7), 2048 x 11008 -> 4096 185.8 us
+// (321.3), 1 x 4096 -> 11008 36.8 us (54.8), 64 x 512 -> 512 5.5 us (6.3), 2048 x
+// 512 -> 8192 27.4 us (34.9), 2048 x 256 -> 8192 20.0 us (23.2). Only at one group,
+// and at two with few tokens, does the former still lead (64 x 128 -> 128 4.1 us
+// against 3.6, 64 x 256 -> 8192 5.7 against 5.3).
 //
 // TMEM (512 columns per CTA): P0, P1, P2 [0, 384), 4 A stages of 32 columns.
 //
-// Warp roles per CTA (32 warps of 64 registers, with 56 / 92 bytes of spill stores / loads; 48 after the start for
+// Warp roles per CTA (32 warps of 64 registers, with 60 / 96 bytes of spill stores / loads; 48 after the start for
 // warps 0-15, 80 for the scalers):
 //   warp 0       TMEM allocation; in the leader CTA, an elected lane issues the MMAs
 //   warps 1-3    stage the windows of s, z and R (cp.async)
@@ -110,7 +111,9 @@ constexpr int kWinW = 2 * kWinRows + kWinR;        // a tile's last window: its 
 constexpr int kWinBytes = kWinW + GBN * 4;
 
 constexpr int kGOffWin = kGStages * kGBStage;
-constexpr int kGOffBars = kGOffWin + 2 * kWinBytes;
+constexpr int kGOutBytes = 32 * 64;      // a scaler warp's buffer for its outputs' way out
+constexpr int kGOffOut = kGOffWin + 2 * kWinBytes;
+constexpr int kGOffBars = kGOffOut + kGScWarps * kGOutBytes;
 constexpr int kGNumBars = 2 * kGStages + 2 * kGBufs + 4;
 constexpr int kGOffMisc = kGOffBars + kGNumBars * 8;
 constexpr int kGUsed = kGOffMisc + 64 + 1024;
@@ -509,7 +512,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
         w ^= 1;
         if (w == 0) wphase ^= 1;
       }
-      if (ok) {
+      if (ok && warp_on && n0 + kGScCols <= p.N) {
+        // Through the warp's buffer, 64 bytes of a row at a time, so that four lanes store one row's 64 bytes: a lane
+        // per row touches 32 lines with each store (2 k cycles a tile: 2048 x 512 -> 8192 32.2 us, now 27.4). Piece q of
+        // row r lies at q ^ (r / 2 % 4): no bank conflicts. A ragged edge leaves directly.
+        constexpr int kElem = OUT == OFFQ_F32 ? 4 : 2, kPer = 16 / kElem;
+        const uint32_t buf = base + kGOffOut + (warp - kGFirstSc) * kGOutBytes;
+        const int row0 = m0 + quarter * 32;
+#pragma unroll
+        for (int c = 0; c < kGScCols; c += 4 * kPer) {
+          __syncwarp();  // the buffer has been read
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              float y0, y1;
+              if constexpr (OUT == OFFQ_F32) {
+                unpack2(S2[(c + 4 * q) / 2 + i / 2], y0, y1);
+                v[i] = __float_as_uint((i & 1) == 0 ? y0 : y1);
+              } else {
+                unpack2(S2[(c + 8 * q) / 2 + i], y0, y1);
+                v[i] = pack_out<OUT>(y0, y1);
+              }
+            }
+            sts128(buf + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4), v[0], v[1], v[2], v[3]);
+          }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = 8 * i + (lane >> 2), q = lane & 3;
+            const uint4 v = lds128(buf + r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
+            if (row0 + r < p.T)
+              *reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) +
+                                        (static_cast<int64_t>(row0 + r) * p.ldo + n0 + c + q * kPer) * kElem) = v;
+          }
+        }
+      } else if (ok && warp_on) {
 #pragma unroll
         for (int c = 0; c < kGScCols; c += 8) {
           float y[8];

@@ -509,15 +509,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kXThreads, 1)
           if (async_out) {  // rows past the tokens too: they are not copied out
             uint32_t hv[CW / 2];
 #pragma unroll
-            for (int i = 0; i < CW / 2; ++i) {
-              if (OUT == OFFQ_BF16) {
-                const __nv_bfloat162 v = __floats2bfloat162_rn(y[2 * i], y[2 * i + 1]);
-                hv[i] = *reinterpret_cast<const uint32_t*>(&v);
-              } else {
-                const __half2 v = __floats2half2_rn(y[2 * i], y[2 * i + 1]);
-                hv[i] = *reinterpret_cast<const uint32_t*>(&v);
-              }
-            }
+            for (int i = 0; i < CW / 2; ++i) hv[i] = pack_out<OUT>(y[2 * i], y[2 * i + 1]);
             sts128(orow_s + c * 2, hv[0], hv[1], hv[2], hv[3]);
             sts128(orow_s + c * 2 + 16, hv[4], hv[5], hv[6], hv[7]);
           } else if (row_ok) {

@@ -243,6 +243,17 @@ __device__ __forceinline__ void widen_weight(uint32_t w, uint32_t& lo, uint32_t&
   hi = __funnelshift_r(w, w, 4) & 0x87878787u;
 }
 
+// Two outputs as one 32-bit word of the 16-bit type OUT, round to nearest even.
+template <int OUT>
+__device__ __forceinline__ uint32_t pack_out(float a, float b) {
+  if (OUT == OFFQ_BF16) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  const __half2 v = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // A 16-byte store, with the L2 policy pol unless pol is 0.
 __device__ __forceinline__ void stg_maybe_hint(void* p, uint4 v, uint64_t pol) {
   if (pol != 0)
@@ -271,15 +282,7 @@ __device__ __forceinline__ void store_out(void* out, int64_t off, const float* y
   } else {
     uint32_t p[CW / 2];
 #pragma unroll
-    for (int i = 0; i < CW / 2; ++i) {
-      if (OUT == OFFQ_BF16) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(y[2 * i], y[2 * i + 1]);
-        p[i] = *reinterpret_cast<const uint32_t*>(&h);
-      } else {
-        const __half2 h = __floats2half2_rn(y[2 * i], y[2 * i + 1]);
-        p[i] = *reinterpret_cast<const uint32_t*>(&h);
-      }
-    }
+    for (int i = 0; i < CW / 2; ++i) p[i] = pack_out<OUT>(y[2 * i], y[2 * i + 1]);
     uint16_t* o = static_cast<uint16_t*>(out) + off;
     if (nvalid == CW) {
 #pragma unroll
