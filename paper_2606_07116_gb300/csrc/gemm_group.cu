@@ -22,8 +22,8 @@
 //
 // What bounds it: issue slots of the SM sub-partitions and the chain of one group.
 // Per group a sub-partition has 32 rows x 128 columns to fold (256 cycles of its
-// FMA pipe) among about 770 warp instructions (waits, TMEM and shared-memory loads,
-// conversions, bookkeeping: 3090 per CTA), and the kernel takes about 1150 cycles
+// FMA pipe) among about 780 warp instructions (waits, TMEM and shared-memory loads,
+// conversions, bookkeeping: 3130 per CTA), and the kernel takes about 1130 cycles
 // per group against 296 of MMA (N = 128, A in tensor memory). Hence four
 // scaler warps per sub-partition (the latency of one is three times its issue
 // time), R read while the partial is waited for, s, z and R in shared memory in
